@@ -81,6 +81,9 @@ __device__ void slot_cells_row(const BatchDesc& D, int j)
     for (int k = threadIdx.x; k < nb; k += blockDim.x) {
         const size_t i = (size_t)j * nb + k;
         if (D.mixed) static_cast<float2*>(D.cells)[i] = map_cell_f32(row, row_lo, k, D.lo[j], D.scale[j], nb);
+        else if (D.cm.fbits)
+            static_cast<double2*>(D.cells)[i] =
+                map_cell_fix(edge_left(row, row_lo, k), edge_right(row, row_lo, k), D.cm, j, inv_g);
         else static_cast<double2*>(D.cells)[i] = map_cell_f64(row, row_lo, k, D.lo[j], D.scale[j], inv_g);
     }
 }
@@ -340,6 +343,7 @@ mcubes_status BatchEngine::admit(const mcubes_request& r, long long tag, int* sl
         D.lo[j] = r.lo[j];
         D.scale[j] = r.hi[j] - r.lo[j];
     }
+    if (!mixed_) affine_prepare(r.integrand_id, r.params, d, D.lo, D.scale, g, nb, &fp, &D.cm, &D.jac0);
     D.fam = fp;
     const size_t grid_stride = 2 * (size_t)kDMax * nb, hist_stride = (size_t)kDMax * nb;
     D.grid = (double*)grids_.ptr + grid_stride * slot;

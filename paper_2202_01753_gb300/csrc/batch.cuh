@@ -66,12 +66,22 @@ vsample_batch_kernel(const __grid_constant__ BatchArgs a)
                           sd.fam};
         const uint32_t it = B.it;
         CubeSums acc;
-        if (adjust)
-            sample_cubes<FAM, MIXED, true, NB4, D>(v, cells, hist, seg.c0, seg.c1 - seg.c0, seg.perm_k, 0, 1, it,
-                                                sd.lanes, sd.p, acc);
-        else
-            sample_cubes<FAM, MIXED, false, NB4, D>(v, cells, hist, seg.c0, seg.c1 - seg.c0, seg.perm_k, 0, 1, it,
-                                                 sd.lanes, sd.p, acc);
+        auto sample = [&](auto adj_c, auto fix_c) {
+            sample_cubes<FAM, MIXED, decltype(adj_c)::value, NB4, D, decltype(fix_c)::value>(
+                v, cells, hist, seg.c0, seg.c1 - seg.c0, seg.perm_k, 0, 1, it, sd.lanes, sd.p, acc);
+        };
+        bool done = false;
+        if constexpr (!MIXED && FixFamily<FAM>::kHas) {
+            if (sd.fam.fix) {  // the fixed-point form: uniform over the segment
+                if (adjust) sample(std::true_type{}, std::true_type{});
+                else sample(std::false_type{}, std::true_type{});
+                done = true;
+            }
+        }
+        if (!done) {
+            if (adjust) sample(std::true_type{}, std::false_type{});
+            else sample(std::false_type{}, std::false_type{});
+        }
         block_write_sums(acc, red, a.seg_part + 3 * (size_t)si);
         if (adjust) {
             __syncthreads();

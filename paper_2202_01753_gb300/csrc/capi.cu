@@ -25,15 +25,15 @@ cudaError_t launch_vsample_c0(bool, bool, const VsArgs&, int, size_t, cudaStream
 cudaError_t launch_vsample_discont(bool, bool, const VsArgs&, int, size_t, cudaStream_t);
 cudaError_t launch_vsample_cosmo6(bool, bool, const VsArgs&, int, size_t, cudaStream_t);
 cudaError_t launch_vsample_table(bool, bool, const VsArgs&, int, size_t, cudaStream_t);
-cudaError_t occupancy_const(bool, bool, int, size_t, int*);
-cudaError_t occupancy_gauss(bool, bool, int, size_t, int*);
-cudaError_t occupancy_corner(bool, bool, int, size_t, int*);
-cudaError_t occupancy_osc(bool, bool, int, size_t, int*);
-cudaError_t occupancy_prodpeak(bool, bool, int, size_t, int*);
-cudaError_t occupancy_c0(bool, bool, int, size_t, int*);
-cudaError_t occupancy_discont(bool, bool, int, size_t, int*);
-cudaError_t occupancy_cosmo6(bool, bool, int, size_t, int*);
-cudaError_t occupancy_table(bool, bool, int, size_t, int*);
+cudaError_t occupancy_const(bool, bool, bool, int, size_t, int*);
+cudaError_t occupancy_gauss(bool, bool, bool, int, size_t, int*);
+cudaError_t occupancy_corner(bool, bool, bool, int, size_t, int*);
+cudaError_t occupancy_osc(bool, bool, bool, int, size_t, int*);
+cudaError_t occupancy_prodpeak(bool, bool, bool, int, size_t, int*);
+cudaError_t occupancy_c0(bool, bool, bool, int, size_t, int*);
+cudaError_t occupancy_discont(bool, bool, bool, int, size_t, int*);
+cudaError_t occupancy_cosmo6(bool, bool, bool, int, size_t, int*);
+cudaError_t occupancy_table(bool, bool, bool, int, size_t, int*);
 
 cudaError_t launch_vsample(int family, bool mixed, bool adjust, const VsArgs& a, int grid, size_t smem,
                            cudaStream_t s)
@@ -52,18 +52,18 @@ cudaError_t launch_vsample(int family, bool mixed, bool adjust, const VsArgs& a,
     }
 }
 
-cudaError_t vsample_occupancy(int family, bool mixed, bool adjust, int d, size_t smem, int* blocks)
+cudaError_t vsample_occupancy(int family, bool mixed, bool adjust, bool fix, int d, size_t smem, int* blocks)
 {
     switch (family) {
-    case MCUBES_F_CONST: return occupancy_const(mixed, adjust, d, smem, blocks);
-    case MCUBES_F_GAUSS: return occupancy_gauss(mixed, adjust, d, smem, blocks);
-    case MCUBES_F_CORNER: return occupancy_corner(mixed, adjust, d, smem, blocks);
-    case MCUBES_F_OSC: return occupancy_osc(mixed, adjust, d, smem, blocks);
-    case MCUBES_F_PRODPEAK: return occupancy_prodpeak(mixed, adjust, d, smem, blocks);
-    case MCUBES_F_C0: return occupancy_c0(mixed, adjust, d, smem, blocks);
-    case MCUBES_F_DISCONT: return occupancy_discont(mixed, adjust, d, smem, blocks);
-    case MCUBES_F_COSMO6: return occupancy_cosmo6(mixed, adjust, d, smem, blocks);
-    case MCUBES_F_TABLE: return occupancy_table(mixed, adjust, d, smem, blocks);
+    case MCUBES_F_CONST: return occupancy_const(mixed, adjust, fix, d, smem, blocks);
+    case MCUBES_F_GAUSS: return occupancy_gauss(mixed, adjust, fix, d, smem, blocks);
+    case MCUBES_F_CORNER: return occupancy_corner(mixed, adjust, fix, d, smem, blocks);
+    case MCUBES_F_OSC: return occupancy_osc(mixed, adjust, fix, d, smem, blocks);
+    case MCUBES_F_PRODPEAK: return occupancy_prodpeak(mixed, adjust, fix, d, smem, blocks);
+    case MCUBES_F_C0: return occupancy_c0(mixed, adjust, fix, d, smem, blocks);
+    case MCUBES_F_DISCONT: return occupancy_discont(mixed, adjust, fix, d, smem, blocks);
+    case MCUBES_F_COSMO6: return occupancy_cosmo6(mixed, adjust, fix, d, smem, blocks);
+    case MCUBES_F_TABLE: return occupancy_table(mixed, adjust, fix, d, smem, blocks);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -128,6 +128,7 @@ bool integrand_prepare(int id, const double* p, int np, int d, FamParams* out, c
         if (!std::isfinite(p[i])) return false;
     out->nf = 0;
     out->tabs = nullptr;
+    out->fix = 0;
     if (id == MCUBES_F_TABLE) {
         if (!table_prepare(p, np, d, out, host_tabs, ntabs, dev_tabs)) return false;
         for (int i = 0; i < kParMax; ++i) {
@@ -526,6 +527,13 @@ mcubes_status mcubes_setup(mcubes_ctx* c, int id, const double* params, int npar
         for (int j = 1; j < d; ++j)
             if (lo[j] != lo[0] || hi[j] != hi[0]) return MCUBES_EINVAL;
 
+    // FP64 affine families: the fixed-point form where the box allows it
+    double scale[kDMax], jac0 = jacobian_scale(g, nb, d) * family_jac_factor(id, fp);
+    for (int j = 0; j < d; ++j) scale[j] = hi[j] - lo[j];
+    CellMap cm;
+    std::memset(&cm, 0, sizeof cm);
+    if (!c->mixed) affine_prepare(id, params, d, lo, scale, g, nb, &fp, &cm, &jac0);
+
     // launch shapes
     c->smem_adj = vsample_smem_bytes(c->mixed, true, d, nb, c->hist_d);
     c->smem_noadj = vsample_smem_bytes(c->mixed, false, d, nb, c->hist_d);
@@ -533,8 +541,8 @@ mcubes_status mcubes_setup(mcubes_ctx* c, int id, const double* params, int npar
     MC_CHECK(c, cudaDeviceGetAttribute(&smem_limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
     if (c->smem_adj + 1024 > (size_t)smem_limit) return MCUBES_EINVAL;  // grid + histogram must fit on chip
     int occ_adj = 0, occ_noadj = 0;
-    MC_CHECK(c, vsample_occupancy(id, c->mixed, true, d, c->smem_adj, &occ_adj));
-    MC_CHECK(c, vsample_occupancy(id, c->mixed, false, d, c->smem_noadj, &occ_noadj));
+    MC_CHECK(c, vsample_occupancy(id, c->mixed, true, fp.fix != 0, d, c->smem_adj, &occ_adj));
+    MC_CHECK(c, vsample_occupancy(id, c->mixed, false, fp.fix != 0, d, c->smem_noadj, &occ_noadj));
     if (occ_adj < 1 || occ_noadj < 1) return MCUBES_EINVAL;
     if (c->opts.blocks_per_sm > 0) {
         occ_adj = std::min(occ_adj, c->opts.blocks_per_sm);
@@ -588,14 +596,15 @@ mcubes_status mcubes_setup(mcubes_ctx* c, int id, const double* params, int npar
     philox_round_keys(c->opts.seed, a.rk);
     for (int j = 0; j < d; ++j) {
         a.lo[j] = lo[j];
-        a.scale[j] = hi[j] - lo[j];
+        a.scale[j] = scale[j];
     }
-    a.jac0 = jacobian_scale(g, nb, d) * family_jac_factor(c->fid, fp);
+    a.jac0 = jac0;
     a.phi_scale_f = (float)(1.0 / ((double)g * nb));
     a.nb_f = (float)nb;
     set_moment_scales(a, p);
     a.want_abs = 0;  // an iteration uses the sums of the cube means and variances only
     a.fam = fp;
+    a.cm = cm;
 
     RefineArgs& r = c->rf;
     std::memset(&r, 0, sizeof r);
@@ -610,8 +619,9 @@ mcubes_status mcubes_setup(mcubes_ctx* c, int id, const double* params, int npar
     std::memset(&c->cellbox, 0, sizeof c->cellbox);
     for (int j = 0; j < d; ++j) {
         r.lo[j] = c->cellbox.lo[j] = lo[j];
-        r.scale[j] = c->cellbox.scale[j] = hi[j] - lo[j];
+        r.scale[j] = c->cellbox.scale[j] = scale[j];
     }
+    r.cm = c->cellbox.cm = cm;
     c->cellbox.g = (uint32_t)g;
     c->cellbox.mixed = c->mixed ? 1 : 0;
     r.st = (DevState*)c->state.ptr;

@@ -136,6 +136,54 @@ __device__ __forceinline__ double fx_log(double x)
     return q64_to_double(hi, lo, neg);
 }
 
+// 2^(n/256) e^r for r = rq 2^-62 in [0, ln2/256], rounded once to a double;
+// SCALED: times (jm / 2^63) 2^je, jm in [2^63, 2^64), before the rounding.
+template <bool SCALED>
+__device__ __forceinline__ double fx_exp_tail(int64_t n, uint64_t rq, uint64_t jm, int je)
+{
+    // e^r = e^(q/65536) e^b with q = floor(r 65536) (< 178) and b < 2^-16 (Q62 < 2^46):
+    // e^b = 1 + b + b^2/2 + b^3/6 (+ b^4/24 < 2^-68), b^2 from the top 32 bits of b
+    // (Hb = b in Q48) and b^3 from b^2 and Hb, with 32 x 32-bit products
+    const uint32_t q = (uint32_t)(rq >> 46);
+    const uint64_t B = rq & ((1ull << 46) - 1);
+    const uint32_t Hb = (uint32_t)(B >> 14);
+    const uint64_t sqb = ((uint64_t)Hb * Hb) >> 34;                      // b^2 in Q62 (< 2^30)
+    const uint32_t cub = (uint32_t)((sqb * Hb) >> 48);                   // b^3 in Q62 (< 2^14)
+    const uint64_t eb = (1ull << 62) + B + (sqb >> 1) + __umulhi(cub, q32_inv(6));  // e^b, Q62
+    const uint64_t s = __umul64hi(__ldg(&kExpK16[q]) << 1, eb << 1);     // e^r, Q62
+    // 2^(j/256) e^r in Q62, within [1, 2)
+    const int j = (int)(n & 255);
+    const int k = (int)(n >> 8);
+    const uint64_t P = __umul64hi(__ldg(&kExp2[j]) << 1, s << 1);
+    // assemble 2^k P / 2^62 (rounded to nearest, ties away): P normalised
+    // into [2^62, 2^63), then a normal double (biased exponent eb >= 1) or,
+    // for eb <= 0 (y below about -708.4), the subnormal round(P 2^-(11 - eb))
+    // (a carry into 2^52 is the smallest normal; below 2^-1075 it is +0)
+    uint64_t Pn = P;
+    int be = k + 1023;  // biased exponent
+    if constexpr (SCALED) {
+        Pn = __umul64hi(P << 1, jm);  // Q62, a value in [1, 4)
+        be += je;
+        if (Pn >> 63) {
+            Pn >>= 1;
+            ++be;
+        }
+        if (be >= 2047) return __longlong_as_double(0x7FF0000000000000ll);  // overflow: +inf
+    }
+    if (Pn < ((uint64_t)1 << 62)) {
+        Pn <<= 1;
+        --be;
+    }
+    uint64_t bits;
+    if (be >= 1) {
+        bits = ((uint64_t)be << 52) + (((Pn + (1ull << 9)) >> 10) - (1ull << 52));
+    } else {
+        const int sh = 11 - be;
+        bits = sh < 64 ? (Pn + (1ull << (sh - 1))) >> sh : 0ull;
+    }
+    return __longlong_as_double((long long)bits);
+}
+
 // exp of the double with bits u; SCALED: exp(y) (jm / 2^63) 2^je, jm in
 // [2^63, 2^64), rounded once.  The scaled form keeps the unscaled one's
 // special cases: where exp(y) alone rounds to +0 the result is +0 (as
@@ -191,47 +239,7 @@ __device__ __forceinline__ double fx_exp_bits_t(uint64_t u, uint64_t jm, int je)
         --n;
         rq += (int64_t)kLn2Over256Q62;
     }
-    // e^r = e^(q/65536) e^b with q = floor(r 65536) (< 178) and b < 2^-16 (Q62 < 2^46):
-    // e^b = 1 + b + b^2/2 + b^3/6 (+ b^4/24 < 2^-68), b^2 from the top 32 bits of b
-    // (Hb = b in Q48) and b^3 from b^2 and Hb, with 32 x 32-bit products
-    const uint32_t q = (uint32_t)((uint64_t)rq >> 46);
-    const uint64_t B = (uint64_t)rq & ((1ull << 46) - 1);
-    const uint32_t Hb = (uint32_t)(B >> 14);
-    const uint64_t sqb = ((uint64_t)Hb * Hb) >> 34;                      // b^2 in Q62 (< 2^30)
-    const uint32_t cub = (uint32_t)((sqb * Hb) >> 48);                   // b^3 in Q62 (< 2^14)
-    const uint64_t eb = (1ull << 62) + B + (sqb >> 1) + __umulhi(cub, q32_inv(6));  // e^b, Q62
-    const uint64_t s = __umul64hi(__ldg(&kExpK16[q]) << 1, eb << 1);     // e^r, Q62
-    // 2^(j/256) e^r in Q62, within [1, 2)
-    const int j = (int)(n & 255);
-    const int k = (int)(n >> 8);
-    const uint64_t P = __umul64hi(__ldg(&kExp2[j]) << 1, s << 1);
-    // assemble 2^k P / 2^62 (rounded to nearest, ties away): P normalised
-    // into [2^62, 2^63), then a normal double (biased exponent eb >= 1) or,
-    // for eb <= 0 (y below about -708.4), the subnormal round(P 2^-(11 - eb))
-    // (a carry into 2^52 is the smallest normal; below 2^-1075 it is +0)
-    uint64_t Pn = P;
-    int be = k + 1023;  // biased exponent
-    if constexpr (SCALED) {
-        Pn = __umul64hi(P << 1, jm);  // Q62, a value in [1, 4)
-        be += je;
-        if (Pn >> 63) {
-            Pn >>= 1;
-            ++be;
-        }
-        if (be >= 2047) return __longlong_as_double(0x7FF0000000000000ll);  // overflow: +inf
-    }
-    if (Pn < ((uint64_t)1 << 62)) {
-        Pn <<= 1;
-        --be;
-    }
-    uint64_t bits;
-    if (be >= 1) {
-        bits = ((uint64_t)be << 52) + (((Pn + (1ull << 9)) >> 10) - (1ull << 52));
-    } else {
-        const int sh = 11 - be;
-        bits = sh < 64 ? (Pn + (1ull << (sh - 1))) >> sh : 0ull;
-    }
-    return __longlong_as_double((long long)bits);
+    return fx_exp_tail<SCALED>(n, (uint64_t)rq, jm, je);
 }
 
 __device__ __forceinline__ double fx_exp_bits(uint64_t u) { return fx_exp_bits_t<false>(u, 0, 0); }
@@ -248,6 +256,102 @@ __device__ __forceinline__ double fx_exp_neg_scaled(double v, uint64_t jm, int j
 __device__ __forceinline__ double fx_exp_neg(double v)
 {
     return fx_exp_bits((uint64_t)__double_as_longlong(v) ^ 0x8000000000000000ull);
+}
+
+// exp(-v) (NEG) or exp(v) of the non-negative fixed-point v = q 2^-fq (fq in
+// 43..62, v < 2^(64 - fq)), times (jm / 2^63) 2^je, rounded once.  v < 746 is
+// split at n ln2/256 with n = floor(v 256/ln2) by one 64-bit high multiply
+// (one more for NEG, so that the remainder of -v is non-negative); the rest
+// is the exponential's own tail.  No conversion to a double on the way in:
+// the FP64 kernels' exponents are sums of fixed-point terms.
+template <bool NEG>
+__device__ __forceinline__ double fx_exp_fixed(uint64_t q, int fq, uint64_t jm, int je)
+{
+    if ((q >> fq) >= 746u) {
+        if constexpr (NEG) return 0.0;  // exp(-v) rounds to +0
+        else return __longlong_as_double(0x7FF0000000000000ll);
+    }
+    const uint64_t H = __umul64hi(q, k256OverLn2Q55);  // v 256/ln2, Q(fq - 9)
+    uint32_t n = (uint32_t)(H >> (fq - 9));
+    if constexpr (NEG) ++n;
+    // n ln2/256 in Q62 (its low 64 bits) from ln2/256 in Q115 = Hi 2^64 + Lo
+    const uint64_t p0 = (uint64_t)n * (uint32_t)kLn2Over256Q115Lo;
+    const uint64_t p1 = (uint64_t)n * (uint32_t)(kLn2Over256Q115Lo >> 32) + (p0 >> 32);  // n Lo / 2^32
+    const uint64_t top = (p1 >> 32) + (uint64_t)n * kLn2Over256Q115Hi;                  // n C in Q51
+    const uint64_t L = (top << 11) + (((p1 & 0xFFFFFFFFull) + (1ull << 20)) >> 21);
+    const uint64_t v = q << (62 - fq);
+    int64_t m = NEG ? -(int64_t)n : (int64_t)n;
+    int64_t rq = (int64_t)(NEG ? L - v : v - L);
+    if (rq < 0) {  // n off by one at a multiple of ln2/256
+        --m;
+        rq += (int64_t)kLn2Over256Q62;
+    }
+    return fx_exp_tail<true>(m, (uint64_t)rq, jm, je);
+}
+
+// First approximation of 1/x, x in [1, 2): 23 bits suffice.
+__device__ __forceinline__ float rcp_seed(float x)
+{
+#ifdef __CUDA_ARCH__
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+#else
+    return 1.0f / x;
+#endif
+}
+
+// 2^64 / x for x = m 2^-63 in [1, 2), by two Newton-Raphson steps y (2 - x y)
+// in fixed point from a single-precision seed kept below 1/x, so that every
+// residual is non-negative: relative error below 2^-60.  Returns a value in
+// [2^63, 2^64): 1/x as Q64.
+__device__ __forceinline__ uint64_t fx_recip(uint64_t m)
+{
+    const float xf = (float)(uint32_t)(m >> 40) * 1.1920928955078125e-07f;  // 24 bits, in [1, 2)
+    // below 1/x by at most 2^-20: the argument was cut by < 2^-23, the seed and
+    // the product are within 2^-22, and 2^-20.9 is taken off
+    const uint32_t y0 = (uint32_t)(rcp_seed(xf) * 4294965148.0f);
+    const uint64_t e0 = (1ull << 63) - __umul64hi(m, (uint64_t)y0 << 32);       // 1 - x y0, Q63 (< 2^43)
+    const uint64_t y1 = ((uint64_t)y0 << 32) + (((uint64_t)y0 * (uint32_t)(e0 >> 11)) >> 20);  // Q64
+    const uint64_t e1 = (1ull << 63) - __umul64hi(m, y1);                       // Q63 (< 2^24)
+    const uint64_t y2 = y1 + (((y1 >> 32) * (uint64_t)(uint32_t)e1) >> 31);
+    return y2 < (1ull << 63) ? (1ull << 63) : y2;  // x next to 2: the truncations may fall short of 1/2
+}
+
+// cos(2 pi t) for the fraction of a turn t = a 2^-64: sign and magnitude, the
+// magnitude as Q63 (up to 2^63).  The quadrant is a's top two bits (odd
+// ones take the complement, cos(pi/2 - y) = sin y); within a quarter turn y
+// = y_j + delta with y_j = (pi/2) j/256 from the table and delta in [0,
+// pi/512): cos y = c_j cos(delta) - s_j sin(delta), the two series cut at
+// delta^6/720 and delta^5/120 (next terms < 2^-63).  Absolute error < 2^-60.
+__device__ __forceinline__ uint64_t fx_cos_turns(uint64_t a, bool* neg)
+{
+    const uint32_t quad = (uint32_t)(a >> 62);
+    *neg = quad == 1u || quad == 2u;
+    uint64_t x = a << 2;
+    if (quad & 1u) x = ~x;
+    const int j = (int)(x >> 56);
+#ifdef __CUDA_ARCH__
+    const ulonglong2 tv = __ldg(reinterpret_cast<const ulonglong2*>(&kCosSin[j]));
+    const uint64_t c = tv.x, s = tv.y;
+#else
+    const uint64_t c = kCosSin[j].c, s = kCosSin[j].s;
+#endif
+    const uint64_t D = __umul64hi((x & 0xFFFFFFFFFFFFFFull) << 7, kHalfPiQ63);  // delta, Q70 (< 2^62.7)
+    const uint64_t D2 = __umul64hi(D, D);                                        // delta^2, Q76 (< 2^61.4)
+    const uint32_t h = (uint32_t)(D2 >> 32);                                     // Q44 (< 2^29.4)
+    // 1 - cos delta = delta^2 (1/2 - delta^2 (1/24 - delta^2/720)), Q76
+    const uint32_t k4 = 2863311531u - __umulhi(h, 23302u);                       // 1/24 - delta^2/720, Q36
+    const uint32_t b = (uint32_t)(((uint64_t)h * k4) >> 29);                     // delta^2 k4, Q51 (< 2^32)
+    const uint64_t u = (D2 >> 1) - (((uint64_t)h * b) >> 19);
+    // sin delta = delta (1 - (delta^2/6 - delta^4/120)), Q70
+    const uint64_t d4 = (uint64_t)h * h;                                         // delta^4, Q88
+    const uint64_t e = __umul64hi(D2, 0x2AAAAAAAAAAAAAABull)                     // delta^2/6, Q76
+                       - ((uint64_t)__umulhi((uint32_t)(d4 >> 28), 35791394u) << 16);  // delta^4/120: Q60 -> Q76
+    const uint64_t sd = D - (__umul64hi(D, e << 4) >> 16);                       // e in Q80: D e in Q86 -> Q70
+    const uint64_t cu = __umul64hi(c, u), ss = __umul64hi(s, sd);                // Q75, Q69
+    const uint64_t r = c - (cu >> 12) - (ss >> 6);
+    return r > (1ull << 63) ? 0ull : r;                                          // rounding below 0 next to a zero
 }
 
 // Single-precision cosine for the mixed-precision kernels: x = k pi/2 + r

@@ -130,6 +130,22 @@ __device__ __forceinline__ void int_prod_mul(IntProd& p, double v)
     p.e += f.e + (int)top;
 }
 
+__device__ __forceinline__ IntProd int_prod_mul2(const IntProd& a, const IntProd& b)
+{
+    const uint64_t H = __umul64hi(a.m, b.m);
+    const uint64_t top = H >> 63;
+    return IntProd{top ? H : H << 1, a.e + b.e + (int)top};
+}
+
+// v 2^-f for v > 0
+__device__ __forceinline__ IntProd int_prod_of_fixed(uint64_t v, int f)
+{
+    const int lz = __clzll((long long)v);
+    return IntProd{v << lz, 63 - lz - f};
+}
+
+__device__ __forceinline__ IntProd int_prod_recip(const IntProd& p) { return IntProd{fx::fx_recip(p.m), -1 - p.e}; }
+
 __device__ __forceinline__ double int_prod_value(const IntProd& p)
 {
     // rounded to 53 bits (2^53 after a carry); m + 2^10 could wrap around
@@ -166,6 +182,31 @@ __device__ __forceinline__ double2 map_cell_f64(const double* row, const double*
     double xl, xw;
     map_cell(row, row_lo, k, lo, scale, &xl, &xw);
     return make_double2(xl, xw * inv_g);
+}
+
+// Map cell of the fixed-point form: (t at the left edge as an integer with
+// m.fbits fraction bits, t width / g as a double).
+__device__ __forceinline__ double2 map_cell_fix(DD left, DD right, const CellMap& m, int j, double inv_g)
+{
+    const DD wd = dd_add(right, DD{-left.hi, -left.lo});
+    const double w = (m.b[j] * (wd.hi + wd.lo)) * inv_g;
+    // b left in two parts, each converted to an integer by itself: short
+    // dependent chains (a dependent FP64 instruction takes 66 cycles)
+    const double sc = __longlong_as_double((long long)(1023 + m.fbits) << 52);  // 2^fbits
+    const double p = __dmul_rn(m.b[j], left.hi);
+    const double e = fma(m.b[j], left.lo, fma(m.b_lo[j], left.hi, __fma_rn(m.b[j], left.hi, -p)));
+    const long long L = m.a[j] + __double2ll_rn(p * sc) + __double2ll_rn(e * sc);
+    return make_double2(__longlong_as_double(L), w);
+}
+
+__device__ __forceinline__ DD edge_right(const double* row, const double* row_lo, uint32_t k)
+{
+    return DD{row[k], row_lo[k]};
+}
+
+__device__ __forceinline__ DD edge_left(const double* row, const double* row_lo, uint32_t k)
+{
+    return k ? DD{row[k - 1], row_lo[k - 1]} : DD{0.0, 0.0};
 }
 
 __device__ __forceinline__ float2 map_cell_f32(const double* row, const double* row_lo, uint32_t k, double lo,
@@ -527,6 +568,136 @@ template <typename R> struct Family<MCUBES_F_TABLE, R> {
             else prod *= TabOps<R>::interp2(T, xa, sel(s, f.tb[q]));
         }
         return prod;
+    }
+};
+
+// ---------------------------------------------------------------------------
+// Fixed-point form of the FP64 affine families.  The integrand reads each
+// coordinate only through t_j = s_j (x_j - o_j) (plus, for DISCONT, a
+// threshold on it), so the map cells hold t_j instead of x_j: the left edge
+// as a 64-bit integer with f fraction bits and the width as a double, and a
+// sample's t_j is one 64-bit high multiply (width significand x g phi's exact
+// numerator), a shift and an addition.  The sums over the axes, the
+// exponential, reciprocal or cosine and the Jacobian's product stay in
+// integers and F = f J is rounded to a double once: no FP64 instruction
+// before the moments and the histogram.  GB300 issues 2 FP64 instructions per
+// clock per SM against 64 integer ones, and the double-precision form of
+// these kernels kept that pipe 80% busy (its practical limit) on 47-100
+// warp instructions per sample.  Adjusting passes of 9.65e6 samples at d = 6,
+// before and with this form: GAUSS 779 -> 392 us, CORNER 676 -> 357, OSC (f_A)
+// 781 -> 336, PRODPEAK 1224 -> 420, C0 879 -> 366, DISCONT 651 -> 360; what is
+// left on the FP64 pipe is the histogram's additions.  t_j's error is 2^-f absolute, f =
+// 57..63 (affine.cu keeps the range of t_j small enough for that, or the
+// double-precision form is used): below the rounding of x itself.
+// Scales: GAUSS t = (x - mu)/(sigma sqrt 2), sum of t^2; C0 t = c (x - w),
+// sum of |t|; DISCONT, CORNER t = a (x - lo); OSC t = a x / (2 pi) in turns,
+// whole turns dropped by the wrap-around; PRODPEAK t = c (x - w), f = prod
+// c^2 / (1 + t^2).  Constant factors are part of the Jacobian's.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint64_t abs_u64(int64_t t) { return t < 0 ? 0ull - (uint64_t)t : (uint64_t)t; }
+
+// t^2 for |t| < 2^63 with f fraction bits: 2 f - 62 fraction bits
+__device__ __forceinline__ uint64_t sq_fixed(int64_t t)
+{
+    const uint64_t a = abs_u64(t) << 1;
+    return __umul64hi(a, a);
+}
+
+template <int FAM> struct FixFamily { static constexpr bool kHas = false; };
+
+struct FixSum {
+    uint64_t q;
+};
+
+template <> struct FixFamily<MCUBES_F_GAUSS> {
+    static constexpr bool kHas = true;
+    using S = FixSum;
+    __device__ static void begin(S& s, const FamParams& f) { s.q = f.fu[kDMax]; }
+    __device__ static void add(S& s, int, int64_t t, const FamParams&) { s.q += sq_fixed(t); }
+    template <int D> __device__ static double end(const S& s, const FamParams& f, const IntProd& jp)
+    {
+        return fx::fx_exp_fixed<true>(s.q, f.fq, jp.m, jp.e);
+    }
+};
+
+template <> struct FixFamily<MCUBES_F_C0> {
+    static constexpr bool kHas = true;
+    using S = FixSum;
+    __device__ static void begin(S& s, const FamParams&) { s.q = 0; }
+    __device__ static void add(S& s, int, int64_t t, const FamParams&) { s.q += abs_u64(t); }
+    template <int D> __device__ static double end(const S& s, const FamParams& f, const IntProd& jp)
+    {
+        return fx::fx_exp_fixed<true>(s.q, f.fq, jp.m, jp.e);
+    }
+};
+
+template <> struct FixFamily<MCUBES_F_DISCONT> {
+    static constexpr bool kHas = true;
+    struct S {
+        uint64_t q;
+        bool out;
+    };
+    __device__ static void begin(S& s, const FamParams&)
+    {
+        s.q = 0;
+        s.out = false;
+    }
+    __device__ static void add(S& s, int j, int64_t t, const FamParams& f)
+    {
+        s.out |= (uint64_t)t >= f.fu[j];
+        s.q += (uint64_t)t;
+    }
+    template <int D> __device__ static double end(const S& s, const FamParams& f, const IntProd& jp)
+    {
+        return s.out ? 0.0 : fx::fx_exp_fixed<false>(s.q, f.fq, jp.m, jp.e);
+    }
+};
+
+template <> struct FixFamily<MCUBES_F_CORNER> {
+    static constexpr bool kHas = true;
+    using S = FixSum;
+    __device__ static void begin(S& s, const FamParams& f) { s.q = f.fu[kDMax]; }
+    __device__ static void add(S& s, int, int64_t t, const FamParams&) { s.q += (uint64_t)t; }
+    template <int D> __device__ static double end(const S& s, const FamParams& f, const IntProd& jp)
+    {
+        // t^-(D+1) J by repeated squaring of 1/t
+        IntProd b = int_prod_recip(int_prod_of_fixed(s.q, f.fq)), r = jp;
+#pragma unroll
+        for (uint32_t e = D + 1; e; e >>= 1) {
+            if (e & 1u) r = int_prod_mul2(r, b);
+            if (e > 1u) b = int_prod_mul2(b, b);
+        }
+        return int_prod_value(r);
+    }
+};
+
+template <> struct FixFamily<MCUBES_F_OSC> {
+    static constexpr bool kHas = true;
+    using S = FixSum;
+    __device__ static void begin(S& s, const FamParams& f) { s.q = f.fu[kDMax]; }
+    __device__ static void add(S& s, int, int64_t t, const FamParams&) { s.q += (uint64_t)t; }
+    template <int D> __device__ static double end(const S& s, const FamParams& f, const IntProd& jp)
+    {
+        bool neg;
+        const uint64_t v = fx::fx_cos_turns(s.q << (64 - f.fq), &neg);
+        if (v == 0) return 0.0;
+        const double F = int_prod_value(int_prod_mul2(jp, int_prod_of_fixed(v, 63)));
+        return neg ? -F : F;
+    }
+};
+
+template <> struct FixFamily<MCUBES_F_PRODPEAK> {
+    static constexpr bool kHas = true;
+    using S = IntProd;
+    __device__ static void begin(S& s, const FamParams&) { s = IntProd{1ull << 63, 0}; }
+    __device__ static void add(S& s, int j, int64_t t, const FamParams& f)
+    {
+        // the squares are cut, by half a last place on average: every other axis takes one back
+        s = int_prod_mul2(s, int_prod_of_fixed((1ull << f.fq) + (uint64_t)(j & 1) + sq_fixed(t), f.fq));
+    }
+    template <int D> __device__ static double end(const S& s, const FamParams&, const IntProd& jp)
+    {
+        return int_prod_value(int_prod_mul2(jp, int_prod_recip(s)));
     }
 };
 

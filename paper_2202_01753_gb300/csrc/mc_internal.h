@@ -76,6 +76,23 @@ struct FamParams {
     int nf;
     int tid[kTabFactorsMax], ta[kTabFactorsMax], tb[kTabFactorsMax];
     const TableDesc* tabs;   // device array of the context's tables
+    // fixed-point form of the FP64 affine families (affine_prepare in affine.cu):
+    // 0 where it does not apply
+    int fix;
+    int fsg;                 // left shift that brings g phi's numerator (< g 2^33) to the top of 64 bits
+    int ftsh;                // a cell width of binary exponent e moves the product right by ftsh - e
+    int fq;                  // fraction bits of the integrand's running sum
+    uint64_t fu[kDMax + 1];  // DISCONT: thresholds; [kDMax]: start of the running sum
+};
+
+// Cells of the fixed-point form: coordinate t = a + b x (x the unit-cube edge)
+// with fbits fraction bits (0: cells in the box's coordinates); b is a
+// double-double.  Sums wrap around 2^64 (OSC: t in turns, whole ones do not
+// matter).
+struct CellMap {
+    long long a[kDMax];
+    double b[kDMax], b_lo[kDMax];
+    int fbits, pad;
 };
 
 // Arguments of one sampling launch (Alg. 3).  Passed by value as a
@@ -108,6 +125,7 @@ struct VsArgs {
     float inv_p_f, inv_var_den_f;  // the same in single precision (mixed)
     uint32_t want_abs;             // part[2] (sums of |cube mean|) wanted: the sampling-pass calls
     FamParams fam;
+    CellMap cm;                    // fam.fix: the cells' coordinates (blocks that build their own cells)
 };
 
 // ---------------------------------------------------------------------------
@@ -129,6 +147,7 @@ struct BatchDesc {
     double lo[kDMax];
     double scale[kDMax];
     FamParams fam;
+    CellMap cm;                 // fam.fix: the cells' coordinates
     double* grid;               // [d][nb] edge high parts, then [d][nb] low parts
     void* cells;                // [d][nb] map cells of the grid (double2 in FP64, float2 in mixed), rebuilt
                                 // by the refinement after each rebin
@@ -195,6 +214,7 @@ struct RefineArgs {
     double* hist_acc;         // [hist_d][nb] histogram of the sampling pass; read, then cleared
     void* cells_g;            // [d][nb] map cells, rebuilt for every rebinned axis (null: none kept)
     double lo[kDMax], scale[kDMax];
+    CellMap cm;               // cm.fbits > 0: cells of the fixed-point form
     uint32_t g;
     int mixed;
     DevState* st;
@@ -209,6 +229,7 @@ struct RefineArgs {
 // The box and format of the map cells (cells_kernel).
 struct CellBox {
     double lo[kDMax], scale[kDMax];
+    CellMap cm;
     uint32_t g;
     int mixed;
 };
@@ -219,7 +240,13 @@ cudaError_t launch_cells(const double* grid, const double* grid_lo, const CellBo
 cudaError_t launch_vsample(int family, bool mixed, bool adjust, const VsArgs& a, int grid,
                            size_t smem, cudaStream_t s);
 size_t vsample_smem_bytes(bool mixed, bool adjust, int d, int nb, int hist_d);
-cudaError_t vsample_occupancy(int family, bool mixed, bool adjust, int d, size_t smem, int* blocks_per_sm);
+cudaError_t vsample_occupancy(int family, bool mixed, bool adjust, bool fix, int d, size_t smem, int* blocks_per_sm);
+// Decides whether an FP64 integrand takes the fixed-point form (affine.cu) on
+// the box lo + scale [0, 1]^d and fills its constants (fp's fixed-point
+// fields, the cells' coordinates, the Jacobian's constant); fp->fix = 0 and
+// *jac0 untouched where it does not.
+void affine_prepare(int id, const double* params, int d, const double* lo, const double* scale, long long g, int nb,
+                    FamParams* fp, CellMap* cm, double* jac0);
 uint64_t cube_permutation(uint64_t n);
 // Raises a kernel's dynamic shared-memory limit on the current device to at
 // least smem bytes (never lowers it, so that contexts of different sizes can

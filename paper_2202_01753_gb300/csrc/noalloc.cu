@@ -91,6 +91,11 @@ extern "C" mcubes_status mcubes_sample_range_noalloc(
         double* hist_acc = reinterpret_cast<double*>(scratch + kPartBytes);
         double* grid_lo = reinterpret_cast<double*>(scratch + kPartBytes + kHistBytes);
 
+        double scale[kDMax], jac0 = jacobian_scale(g, nbins, d) * family_jac_factor(integrand_id, fp);
+        for (int j = 0; j < d; ++j) scale[j] = hi[j] - lo[j];
+        CellMap cm;
+        std::memset(&cm, 0, sizeof cm);
+        if (!mixed) affine_prepare(integrand_id, params, d, lo, scale, g, nbins, &fp, &cm, &jac0);
         const size_t smem = vsample_smem_bytes(mixed, adj, d, nbins, d);
         const size_t smem_other = vsample_smem_bytes(mixed, !adj, d, nbins, d);
         int smem_limit = 0, sms = 0, occ = 0, occ_other = 0;
@@ -100,8 +105,8 @@ extern "C" mcubes_status mcubes_sample_range_noalloc(
             break;
         }
         if (smem + 1024 > (size_t)smem_limit) { st = MCUBES_EINVAL; break; }
-        if (vsample_occupancy(integrand_id, mixed, adj, d, smem, &occ) != cudaSuccess || occ < 1 ||
-            vsample_occupancy(integrand_id, mixed, !adj, d, smem_other, &occ_other) != cudaSuccess) {
+        if (vsample_occupancy(integrand_id, mixed, adj, fp.fix != 0, d, smem, &occ) != cudaSuccess || occ < 1 ||
+            vsample_occupancy(integrand_id, mixed, !adj, fp.fix != 0, d, smem_other, &occ_other) != cudaSuccess) {
             st = MCUBES_ECUDA;
             break;
         }
@@ -138,14 +143,15 @@ extern "C" mcubes_status mcubes_sample_range_noalloc(
         philox_round_keys(seed, a.rk);
         for (int j = 0; j < d; ++j) {
             a.lo[j] = lo[j];
-            a.scale[j] = hi[j] - lo[j];
+            a.scale[j] = scale[j];
         }
-        a.jac0 = jacobian_scale(g, nbins, d) * family_jac_factor(integrand_id, fp);
+        a.jac0 = jac0;
         a.phi_scale_f = (float)(1.0 / ((double)g * nbins));
         a.nb_f = (float)nbins;
         set_moment_scales(a, p);
         a.want_abs = 1;  // the pass reports the sum of |cube mean|
         a.fam = fp;
+        a.cm = cm;
 
         // the grid's low parts must read as zero and the histogram accumulator
         // start empty; the partials are overwritten

@@ -111,9 +111,13 @@ static __device__ void rebin_axis_cluster(const RefineArgs& a, int ax, int rank,
                                   cluster.map_shared_rank(sEl, rank - 1)[chunk - 1]};
         for (int r = 0; r < rows; ++r) {
             const int j = ax + r;
+            const size_t i = (size_t)j * nb + k;
+            if (a.cm.fbits) {
+                static_cast<double2*>(a.cells_g)[i] = map_cell_fix(left, right, a.cm, j, inv_g);
+                continue;
+            }
             double xl, xw;
             map_cell_edges(left, right, a.lo[j], a.scale[j], &xl, &xw);
-            const size_t i = (size_t)j * nb + k;
             if (a.mixed) static_cast<float2*>(a.cells_g)[i] = make_float2((float)xl, (float)(xw * (double)nb));
             else static_cast<double2*>(a.cells_g)[i] = make_double2(xl, xw * inv_g);
         }
@@ -186,7 +190,7 @@ __global__ void combine_shards_kernel(const double* gathered, int nranks, int le
 }
 
 // Map cells of the whole grid (set-up, and after the grid is replaced).
-__global__ void cells_kernel(const double* grid, const double* grid_lo, CellBox box, int d, int nb, void* out)
+__global__ void cells_kernel(const double* grid, const double* grid_lo, const __grid_constant__ CellBox box, int d, int nb, void* out)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= d * nb) return;
@@ -194,6 +198,9 @@ __global__ void cells_kernel(const double* grid, const double* grid_lo, CellBox 
     const double* row = grid + (size_t)j * nb;
     const double* row_lo = grid_lo + (size_t)j * nb;
     if (box.mixed) static_cast<float2*>(out)[i] = map_cell_f32(row, row_lo, k, box.lo[j], box.scale[j], nb);
+    else if (box.cm.fbits)
+        static_cast<double2*>(out)[i] =
+            map_cell_fix(edge_left(row, row_lo, k), edge_right(row, row_lo, k), box.cm, j, 1.0 / (double)box.g);
     else static_cast<double2*>(out)[i] = map_cell_f64(row, row_lo, k, box.lo[j], box.scale[j], 1.0 / (double)box.g);
 }
 

@@ -133,10 +133,11 @@ template <> struct Prec<true> {
 // histogram ([hist_d][nb]).  grid/grid_lo: [d][nb] double-double right
 // edges (unit cube); lo/scale: the box's lower corner and hi - lo; g:
 // sub-cubes per axis.
-template <bool MIXED, bool ADJ, class Arr>
+template <bool MIXED, bool ADJ, bool FIX, class Arr>
 __device__ __forceinline__ void stage_grid(typename Prec<MIXED>::Cell* cells, typename Prec<MIXED>::H* hist,
                                            const double* grid, const double* grid_lo, const Arr& lo,
-                                           const Arr& scale, uint32_t d, uint32_t nb, uint32_t g, uint32_t hist_d)
+                                           const Arr& scale, const CellMap& cm, uint32_t d, uint32_t nb, uint32_t g,
+                                           uint32_t hist_d)
 {
     if constexpr (ADJ)
         for (uint32_t i = threadIdx.x; i < hist_d * nb; i += blockDim.x) hist[i] = typename Prec<MIXED>::H(0);
@@ -144,6 +145,9 @@ __device__ __forceinline__ void stage_grid(typename Prec<MIXED>::Cell* cells, ty
     for (uint32_t i = threadIdx.x; i < d * nb; i += blockDim.x) {
         const uint32_t j = i / nb, k = i - j * nb;
         if constexpr (MIXED) cells[i] = map_cell_f32(grid + j * nb, grid_lo + j * nb, k, lo[j], scale[j], nb);
+        else if constexpr (FIX)
+            cells[i] = map_cell_fix(edge_left(grid + j * nb, grid_lo + j * nb, k),
+                                    edge_right(grid + j * nb, grid_lo + j * nb, k), cm, (int)j, inv_g);
         else cells[i] = map_cell_f64(grid + j * nb, grid_lo + j * nb, k, lo[j], scale[j], inv_g);
     }
 }
@@ -244,17 +248,59 @@ sample_point_rolled(const A& a, const typename Prec<MIXED>::Cell* cells, uint32_
     else return Fam::end(fs, D, a.fam) * jac;
 }
 
+// The same sample in the fixed-point form (FixFamily): the cell holds t at
+// the left edge with f fraction bits and width / g as a double, of value M
+// 2^(e - 63); g phi = num 2^-33, num < g 2^33 shifted to the top of 64 bits by
+// fsg, so t = left + (M num 2^fsg) >> (64 + ftsh - e).
+template <int FAM, int NB4, int DC, class A>
+__device__ __forceinline__ double sample_point_fix(const A& a, const double2* cells, uint32_t c, uint32_t s,
+                                                   uint32_t it, const uint32_t (&nbc)[4 * NB4],
+                                                   uint32_t (&idx)[2 * NB4])
+{
+    using Fam = FixFamily<FAM>;
+    const uint32_t nb = a.nb;
+    uint32_t w[4 * NB4];
+#pragma unroll
+    for (int b = 0; b < NB4; ++b) {
+        const uint4 r = sample_words(a, make_uint4(s, c, it, (uint32_t)b));
+        w[4 * b + 0] = r.x;
+        w[4 * b + 1] = r.y;
+        w[4 * b + 2] = r.z;
+        w[4 * b + 3] = r.w;
+    }
+    typename Fam::S fs;
+    Fam::begin(fs, a.fam);
+    IntProd jp = int_prod_of(a.jac0);
+#pragma unroll
+    for (int j = 0; j < DC; ++j) {
+        const BinPos bp = bin_pos(w[j], nbc[j], nb, a.g, a.gmagic);
+        const uint32_t flat = (uint32_t)j * nb + bp.k;
+        const double2 cell = cells[flat];
+        const IntProd wd = int_prod_of(cell.y);
+        const uint64_t num = (((uint64_t)((bp.r << 1) | bp.ahi) << 32) | (uint64_t)bp.alo) << a.fam.fsg;
+        const uint64_t H = __umul64hi(wd.m, num);
+        const uint32_t sh = (uint32_t)(a.fam.ftsh - wd.e);  // >= 0; beyond 63 for the narrowest bins
+        const int64_t t = __double_as_longlong(cell.x) + (int64_t)(sh < 64u ? H >> sh : 0ull);
+        jp = int_prod_mul2(jp, wd);
+        Fam::add(fs, j, t, a.fam);
+        if (j & 1) idx[j >> 1] |= flat << 16;
+        else idx[j >> 1] = flat;
+    }
+    return Fam::template end<DC>(fs, a.fam, jp);
+}
+
 // One sample: random words -> exact bin position -> map -> integrand.
 // Returns F = f(x) * J and leaves the flat histogram index of every axis in
 // idx (16 bits each, two per word).  A provides d, nb, g, gmagic, jac0 ((g nb)^d), phi_scale_f
 // (1/(g nb)), hist_d and fam, and sample_words(a, counter) its Philox block.
-template <int FAM, bool MIXED, int NB4, int DC = 0, class A>
+template <int FAM, bool MIXED, int NB4, int DC, bool FIX, class A>
 __device__ __forceinline__ typename Prec<MIXED>::R
 sample_point(const A& a, const typename Prec<MIXED>::Cell* cells, uint32_t c, uint32_t s, uint32_t it,
              const uint32_t (&nbc)[4 * NB4], uint32_t (&idx)[2 * NB4])
 {
     using R = typename Prec<MIXED>::R;
     using Fam = Family<FAM, R>;
+    if constexpr (FIX) return sample_point_fix<FAM, NB4, DC>(a, cells, c, s, it, nbc, idx);
     if constexpr (DC > 0 && rolled_axes<FAM, MIXED>()) {
         return sample_point_rolled<FAM, MIXED, NB4, DC>(a, cells, c, s, it, idx);
     }
@@ -321,7 +367,7 @@ struct CubeSums {
 // inv_p = 1/p and inv_var_den = 1/(p (p-1)) (inv_p_f, inv_var_den_f in single
 // precision) and want_abs (whether the sums of |cube mean| are needed: they
 // are reported by the sampling-pass calls, not used by an iteration).
-template <int FAM, bool MIXED, bool ADJ, int NB4, int DC = 0, class A>
+template <int FAM, bool MIXED, bool ADJ, int NB4, int DC, bool FIX, class A>
 __device__ __forceinline__ void sample_cubes(const A& a, const typename Prec<MIXED>::Cell* cells,
                                              typename Prec<MIXED>::H* hist, uint64_t cube_lo, uint64_t ncubes,
                                              uint64_t perm_k, uint64_t group0, uint64_t gstride, uint32_t it,
@@ -379,7 +425,7 @@ __device__ __forceinline__ void sample_cubes(const A& a, const typename Prec<MIX
         if (valid) {
             for (uint32_t s = seg_lane; s < p; s += L) {
                 uint32_t idx[2 * NB4];
-                const R F = sample_point<FAM, MIXED, NB4, DC>(a, cells, c, s, it, nbc, idx);
+                const R F = sample_point<FAM, MIXED, NB4, DC, FIX>(a, cells, c, s, it, nbc, idx);
                 if (n == 0) {
                     K = F;  // the shift: its own term is zero
                 } else if (n == 1) {
@@ -458,7 +504,7 @@ __device__ __forceinline__ void sample_cubes(const A& a, const typename Prec<MIX
 // S2 += dK (2 S1 + n dK), dK = K_t - K: no division) and summed in a fixed
 // order; the block writes (K, S1, S2) to out[0..2] and the refinement
 // combines a cube's blocks the same way.
-template <int FAM, bool MIXED, bool ADJ, int NB4, int DC = 0, class A>
+template <int FAM, bool MIXED, bool ADJ, int NB4, int DC, bool FIX, class A>
 __device__ __forceinline__ void sample_cube_slice(const A& a, const typename Prec<MIXED>::Cell* cells,
                                                   typename Prec<MIXED>::H* hist, uint64_t cube, uint32_t k,
                                                   uint32_t split, uint32_t it, uint32_t p,
@@ -492,7 +538,7 @@ __device__ __forceinline__ void sample_cube_slice(const A& a, const typename Pre
     uint32_t n = 0;
     for (uint32_t s = s_lo + threadIdx.x; s < s_hi; s += blockDim.x) {
         uint32_t idx[2 * NB4];
-        const R F = sample_point<FAM, MIXED, NB4, DC>(a, cells, c, s, it, nbc, idx);
+        const R F = sample_point<FAM, MIXED, NB4, DC, FIX>(a, cells, c, s, it, nbc, idx);
         if (n == 0) {
             K = F;  // the shift: its own term is zero
         } else {
@@ -595,7 +641,7 @@ constexpr int vsample_kernel_min_blocks()
 // constant every per-axis loop is unrolled without guards and the families'
 // dimension-dependent code (the corner family's power) folds (corner8: 21.4
 // -> 17.7 ms per 1e9-call launch against a runtime count).
-template <int FAM, bool MIXED, bool ADJ, int D>
+template <int FAM, bool MIXED, bool ADJ, int D, bool FIX>
 __global__ void __launch_bounds__(vsample_threads(FAM, MIXED, D), vsample_kernel_min_blocks<FAM, MIXED, D>())
 vsample_kernel(const __grid_constant__ VsArgs a)
 {
@@ -621,16 +667,16 @@ vsample_kernel(const __grid_constant__ VsArgs a)
     Cell* cells = reinterpret_cast<Cell*>(smem);
     HT* hist = reinterpret_cast<HT*>(smem + cell_bytes(MIXED) * d * nb);
     if (a.cells_g) stage_cells<MIXED, ADJ>(cells, hist, a.cells_g, d, nb, a.hist_d);
-    else stage_grid<MIXED, ADJ>(cells, hist, a.grid, a.grid_lo, a.lo, a.scale, d, nb, a.g, a.hist_d);
+    else stage_grid<MIXED, ADJ, FIX>(cells, hist, a.grid, a.grid_lo, a.lo, a.scale, a.cm, d, nb, a.g, a.hist_d);
     __syncthreads();
 
     if (a.split > 1) {
-        sample_cube_slice<FAM, MIXED, ADJ, NB4, D>(a, cells, hist, a.cube_begin + blockIdx.x / a.split,
+        sample_cube_slice<FAM, MIXED, ADJ, NB4, D, FIX>(a, cells, hist, a.cube_begin + blockIdx.x / a.split,
                                                 blockIdx.x % a.split, a.split, it, a.p, red,
                                                 a.part + 3 * (size_t)blockIdx.x);
     } else {
         CubeSums acc;
-        sample_cubes<FAM, MIXED, ADJ, NB4, D>(a, cells, hist, a.cube_begin, a.cube_end - a.cube_begin, a.perm_k,
+        sample_cubes<FAM, MIXED, ADJ, NB4, D, FIX>(a, cells, hist, a.cube_begin, a.cube_end - a.cube_begin, a.perm_k,
                                            blockIdx.x, gridDim.x, it, a.lanes, a.p, acc);
         block_write_sums(acc, red, a.part + 3 * (size_t)blockIdx.x);
     }
@@ -646,38 +692,41 @@ vsample_kernel(const __grid_constant__ VsArgs a)
     }
 }
 
-template <int FAM, bool MIXED, bool ADJ>
+template <int FAM, bool MIXED, bool ADJ, bool FIX>
 inline auto vsample_kernel_d(int d)
 {
     using K = void (*)(VsArgs);
     switch (d) {
-    case 1: return (K)vsample_kernel<FAM, MIXED, ADJ, 1>;
-    case 2: return (K)vsample_kernel<FAM, MIXED, ADJ, 2>;
-    case 3: return (K)vsample_kernel<FAM, MIXED, ADJ, 3>;
-    case 4: return (K)vsample_kernel<FAM, MIXED, ADJ, 4>;
-    case 5: return (K)vsample_kernel<FAM, MIXED, ADJ, 5>;
-    case 6: return (K)vsample_kernel<FAM, MIXED, ADJ, 6>;
-    case 7: return (K)vsample_kernel<FAM, MIXED, ADJ, 7>;
-    case 8: return (K)vsample_kernel<FAM, MIXED, ADJ, 8>;
-    case 9: return (K)vsample_kernel<FAM, MIXED, ADJ, 9>;
-    case 10: return (K)vsample_kernel<FAM, MIXED, ADJ, 10>;
-    case 11: return (K)vsample_kernel<FAM, MIXED, ADJ, 11>;
-    default: return (K)vsample_kernel<FAM, MIXED, ADJ, 12>;  // d is checked to be 1..12
+    case 1: return (K)vsample_kernel<FAM, MIXED, ADJ, 1, FIX>;
+    case 2: return (K)vsample_kernel<FAM, MIXED, ADJ, 2, FIX>;
+    case 3: return (K)vsample_kernel<FAM, MIXED, ADJ, 3, FIX>;
+    case 4: return (K)vsample_kernel<FAM, MIXED, ADJ, 4, FIX>;
+    case 5: return (K)vsample_kernel<FAM, MIXED, ADJ, 5, FIX>;
+    case 6: return (K)vsample_kernel<FAM, MIXED, ADJ, 6, FIX>;
+    case 7: return (K)vsample_kernel<FAM, MIXED, ADJ, 7, FIX>;
+    case 8: return (K)vsample_kernel<FAM, MIXED, ADJ, 8, FIX>;
+    case 9: return (K)vsample_kernel<FAM, MIXED, ADJ, 9, FIX>;
+    case 10: return (K)vsample_kernel<FAM, MIXED, ADJ, 10, FIX>;
+    case 11: return (K)vsample_kernel<FAM, MIXED, ADJ, 11, FIX>;
+    default: return (K)vsample_kernel<FAM, MIXED, ADJ, 12, FIX>;  // d is checked to be 1..12
     }
 }
 
+// The kernel of a launch; fix: its fixed-point form (families that have one).
 template <int FAM>
-inline auto vsample_kernel_ptr(bool mixed, bool adjust, int d)
+inline auto vsample_kernel_ptr(bool mixed, bool adjust, bool fix, int d)
 {
-    if (mixed) return adjust ? vsample_kernel_d<FAM, true, true>(d) : vsample_kernel_d<FAM, true, false>(d);
-    return adjust ? vsample_kernel_d<FAM, false, true>(d) : vsample_kernel_d<FAM, false, false>(d);
+    if (mixed) return adjust ? vsample_kernel_d<FAM, true, true, false>(d) : vsample_kernel_d<FAM, true, false, false>(d);
+    if constexpr (FixFamily<FAM>::kHas)
+        if (fix) return adjust ? vsample_kernel_d<FAM, false, true, true>(d) : vsample_kernel_d<FAM, false, false, true>(d);
+    return adjust ? vsample_kernel_d<FAM, false, true, false>(d) : vsample_kernel_d<FAM, false, false, false>(d);
 }
 
 template <int FAM>
 cudaError_t launch_vsample_family(bool mixed, bool adjust, const VsArgs& a, int grid, size_t smem,
                                   cudaStream_t s)
 {
-    auto k = vsample_kernel_ptr<FAM>(mixed, adjust, (int)a.d);
+    auto k = vsample_kernel_ptr<FAM>(mixed, adjust, a.fam.fix != 0, (int)a.d);
     cudaError_t e = raise_smem_limit((const void*)k, smem);
     if (e != cudaSuccess) return e;
     k<<<grid, vsample_threads(FAM, mixed, (int)a.d), smem, s>>>(a);
@@ -685,9 +734,9 @@ cudaError_t launch_vsample_family(bool mixed, bool adjust, const VsArgs& a, int 
 }
 
 template <int FAM>
-cudaError_t occupancy_family(bool mixed, bool adjust, int d, size_t smem, int* blocks)
+cudaError_t occupancy_family(bool mixed, bool adjust, bool fix, int d, size_t smem, int* blocks)
 {
-    auto k = vsample_kernel_ptr<FAM>(mixed, adjust, d);
+    auto k = vsample_kernel_ptr<FAM>(mixed, adjust, fix, d);
     cudaError_t e = raise_smem_limit((const void*)k, smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k, vsample_threads(FAM, mixed, d), smem);
@@ -702,8 +751,8 @@ cudaError_t occupancy_family(bool mixed, bool adjust, int d, size_t smem, int* b
     {                                                                                             \
         return launch_vsample_family<FAM>(mixed, adjust, a, grid, smem, s);                       \
     }                                                                                             \
-    cudaError_t occupancy_##NAME(bool mixed, bool adjust, int d, size_t smem, int* blocks)        \
+    cudaError_t occupancy_##NAME(bool mixed, bool adjust, bool fix, int d, size_t smem, int* blocks) \
     {                                                                                             \
-        return occupancy_family<FAM>(mixed, adjust, d, smem, blocks);                             \
+        return occupancy_family<FAM>(mixed, adjust, fix, d, smem, blocks);                             \
     }                                                                                             \
     }

@@ -23,6 +23,10 @@ floating-point arithmetic", ACM TOMS 15(2), 1989:
   nearest to what remains of pi/2) for a Cody-Waite reduction (Cody and
   Waite, "Software Manual for the Elementary Functions", 1980), and 2/pi.
 
+* cosine of turns: cos and sin of (pi/2) j/256 for j = 0..255 as unsigned Q63
+  integers, side by side (one 16-byte load per lookup); pi/2 as a Q63 integer.
+  1/(2 pi) as the sum of two doubles, for the host's frequencies in turns.
+
 Values are computed with 60-digit mpmath arithmetic and rounded once.
 Run from the repository root: python -m paper_2202_01753_gb300.gen_fx_tables
 """
@@ -111,6 +115,10 @@ def render():
         f"constexpr float kHalfPiF2 = {_f32(hp - _f32(hp))!r}f;",
         f"constexpr float kHalfPiF3 = {_f32(hp - _f32(hp) - _f32(hp - _f32(hp)))!r}f;",
         f"constexpr float kTwoOverPiF = {_f32(2 / mpmath.pi)!r}f;",
+        f"constexpr uint64_t kHalfPiQ63 = 0x{int(mpmath.nint(hp * mpmath.mpf(2) ** 63)):016x}ull;  // pi/2 as Q63",
+        f"constexpr uint64_t k256OverLn2Q55 = 0x{int(mpmath.nint(256 / ln2 * mpmath.mpf(2) ** 55)):016x}ull;  // 256/ln2 as Q55",
+        f"constexpr double kInv2PiHi = {_dd(1 / (2 * mpmath.pi))[0]!r};  // 1/(2 pi) = Hi + Lo",
+        f"constexpr double kInv2PiLo = {_dd(1 / (2 * mpmath.pi))[1]!r};",
         "",
         "// A logarithm table entry: 1/c as Q63 and ln c as Q64, loaded together",
         "struct alignas(16) LogPair {",
@@ -127,6 +135,14 @@ def render():
     inv_d, log_d, exp_k = second_step_tables()
     _pair_table(lines, "// d_k = 1 + k/65536: 1/d_k as Q63 (k = 0: exactly 2^63), ln d_k as Q64", "kLogD", inv_d, log_d)
     _table(lines, "// exp(k/65536) as Q62", "kExpK16", exp_k)
+    mpmath.mp.dps = 60
+    cs = [(int(mpmath.nint(2 ** 63 * mpmath.cos(hp * j / 256))), int(mpmath.nint(2 ** 63 * mpmath.sin(hp * j / 256))))
+          for j in range(256)]
+    lines += ["// A cosine table entry, loaded together", "struct alignas(16) CosPair {", "    uint64_t c, s;", "};", "",
+              "// cos and sin of (pi/2) j/256 as Q63", "__device__ const CosPair kCosSin[256] = {"]
+    for i in range(0, 256, 2):
+        lines.append("    " + " ".join(f"{{0x{a:016x}ull, 0x{b:016x}ull}}," for a, b in cs[i:i + 2]))
+    lines += ["};", ""]
     lines += ["}  // namespace fx", "}  // namespace mc", ""]
     return "\n".join(lines)
 
