@@ -172,11 +172,12 @@ void affine_prepare(int id, const double* params, int d, const double* lo, const
     }
     default: return;
     }
-    // J f0 = prod (nb scale_j) f0 = jac0 prod W_j with W_j = b_j (unit width) (1/g), as the cells hold it
-    const double inv_g = 1.0 / (double)g;
-    HD j0 = fac;
-    for (int j = 0; j < d; ++j)
-        j0 = mul(j0, div(mul(HD{(double)nb, 0.0}, HD{scale[j], 0.0}), mul(HD{b[j].h, 0.0}, HD{inv_g, 0.0})));
+    // J f0 = prod (nb scale_j) f0 = jac0 prod W_j with W_j = (b_j / g) (unit width), as the cells hold it
+    HD j0 = fac, bg[kDMax];
+    for (int j = 0; j < d; ++j) {
+        bg[j] = div(b[j], HD{(double)g, 0.0});
+        j0 = mul(j0, div(mul(HD{(double)nb, 0.0}, HD{scale[j], 0.0}), bg[j]));
+    }
     if (!std::isnormal(j0.h) || !(j0.h > 0.0)) return;
     int lg = 0;  // ceil(log2 g)
     while ((1ll << lg) < g) ++lg;
@@ -184,8 +185,13 @@ void affine_prepare(int id, const double* params, int d, const double* lo, const
     for (int j = 0; j < d; ++j) {
         if (id == MCUBES_F_OSC) a[j] = add(a[j], HD{-std::nearbyint(a[j].h), 0.0});
         cm->a[j] = to_fixed(a[j], f);
-        cm->b[j] = b[j].h;
-        cm->b_lo[j] = b[j].l;
+        cm->b[j] = (uint64_t)to_fixed(b[j], f);
+        int e;  // b / g = m 2^(e - 63), m in [2^63, 2^64): rounded to 61 bits
+        (void)std::frexp(bg[j].h, &e);
+        const uint64_t v = (uint64_t)to_fixed(bg[j], 61 - e);  // 2^60..2^61
+        const int z = __builtin_clzll(v);
+        cm->bg_m[j] = v << z;
+        cm->bg_e[j] = e + 2 - z;  // v 2^(e - 61) = m 2^(e - 61 - z)
     }
     cm->fbits = f;
     fp->fix = 1;

@@ -71,24 +71,16 @@ namespace {
 
 using namespace refine_detail;
 
-// Map cells of one axis of a slot from its grid (block-wide).
-__device__ void slot_cells_row(const BatchDesc& D, int j)
+// Map cell k of axis j of a slot.
+__device__ __forceinline__ void slot_cell(const BatchDesc& D, int j, int k, DD left, DD right, double inv_g)
 {
-    const int nb = (int)D.nb;
-    const double* row = D.grid + (size_t)j * nb;
-    const double* row_lo = D.grid + (size_t)D.d * nb + (size_t)j * nb;
-    const double inv_g = 1.0 / (double)D.g;
-    for (int k = threadIdx.x; k < nb; k += blockDim.x) {
-        const size_t i = (size_t)j * nb + k;
-        if (D.mixed) static_cast<float2*>(D.cells)[i] = map_cell_f32(row, row_lo, k, D.lo[j], D.scale[j], nb);
-        else if (D.cm.fbits)
-            static_cast<double2*>(D.cells)[i] =
-                map_cell_fix(edge_left(row, row_lo, k), edge_right(row, row_lo, k), D.cm, j, inv_g);
-        else static_cast<double2*>(D.cells)[i] = map_cell_f64(row, row_lo, k, D.lo[j], D.scale[j], inv_g);
-    }
+    const size_t i = (size_t)j * D.nb + k;
+    if (D.mixed) static_cast<float2*>(D.cells)[i] = map_cell_f32(left, right, D.lo[j], D.scale[j], D.nb);
+    else if (D.cm.fbits) static_cast<double2*>(D.cells)[i] = map_cell_fix(left, right, D.cm, j);
+    else static_cast<double2*>(D.cells)[i] = map_cell_f64(left, right, D.lo[j], D.scale[j], inv_g);
 }
 
-__device__ void refine_one(const BatchRefineArgs& a, uint32_t j, double* scratch);
+__device__ void refine_one(const BatchRefineArgs& a, uint32_t j, RebinShared& sh);
 
 // Refinement of one iteration of every live integral: block row y handles
 // live integrals y, y + gridDim.y, ...; for integral j, block (axis, row)
@@ -96,15 +88,15 @@ __device__ void refine_one(const BatchRefineArgs& a, uint32_t j, double* scratch
 // the integral's segment partials in order and weighs the iteration.
 __global__ void __launch_bounds__(kRefineThreads) refine_batch_kernel(const __grid_constant__ BatchRefineArgs a)
 {
-    __shared__ double scratch[33];
+    __shared__ RebinShared sh;
     const uint32_t nlive = *a.nlive;
     for (uint32_t j = blockIdx.y; j < nlive; j += gridDim.y) {
-        refine_one(a, j, scratch);
-        __syncthreads();  // scratch is reused by the next integral
+        refine_one(a, j, sh);
+        __syncthreads();  // the shared memory is reused by the next integral
     }
 }
 
-__device__ void refine_one(const BatchRefineArgs& a, uint32_t j, double* scratch)
+__device__ void refine_one(const BatchRefineArgs& a, uint32_t j, RebinShared& sh)
 {
     const uint32_t slot = a.live[j];
     const BatchDesc& D = a.desc[slot];
@@ -134,10 +126,33 @@ __device__ void refine_one(const BatchRefineArgs& a, uint32_t j, double* scratch
         const size_t off = (size_t)ax * nb;
         const size_t elem = a.hist_is_float ? sizeof(float) : sizeof(double);
         const char* parts = static_cast<const char*>(a.seg_hist) + (a.segs[s0].hist_off + off) * elem;
-        rebin_axis(parts, (size_t)d * nb, (int)(s1 - s0), a.hist_is_float != 0, nb, a.alpha, D.grid + off,
-                   D.grid + (size_t)d * nb + off, D.hist + off, &st->error, &st->done, scratch);
-        __syncthreads();  // the axis's new edges are in global memory: rebuild its map cells
-        slot_cells_row(D, ax);
+        const size_t stride = (size_t)d * nb;
+        const int nparts = (int)(s1 - s0);
+        double* grid = D.grid + off;
+        double* grid_lo = D.grid + stride + off;
+        for (int k = threadIdx.x; k < nb; k += kRefineThreads) {
+            // the histogram: the sum of the integral's segments in their order
+            double acc = 0.0;
+            if (a.hist_is_float) {
+                const float* ph = reinterpret_cast<const float*>(parts) + k;
+                for (int b = 0; b < nparts; ++b) acc += (double)ph[b * stride];
+            } else {
+                const double* ph = reinterpret_cast<const double*>(parts) + k;
+                for (int b = 0; b < nparts; ++b) acc += ph[b * stride];
+            }
+            sh.C[k] = acc;
+            sh.B[k] = grid[k];
+            sh.Blo[k] = grid_lo[k];
+            D.hist[off + k] = acc;
+        }
+        if (!rebin_block(sh, nb, a.alpha, &st->error, &st->done)) return;
+        const double inv_g = 1.0 / (double)D.g;
+        for (int k = threadIdx.x; k < nb; k += kRefineThreads) {
+            const DD right = edge_right(sh.B, sh.Blo, k), left = edge_left(sh.B, sh.Blo, k);
+            grid[k] = right.hi;
+            grid_lo[k] = right.lo;
+            slot_cell(D, ax, k, left, right, inv_g);
+        }
     }
 }
 
@@ -160,7 +175,13 @@ __global__ void init_slots_kernel(const BatchDesc* desc, BatchState* st, const u
         D.hist[i] = 0.0;
     }
     __syncthreads();  // the grid is in global memory: build the map cells
-    for (int j = 0; j < d; ++j) slot_cells_row(D, j);
+    const double inv_g = 1.0 / (double)D.g;
+    for (int i = threadIdx.x; i < d * nb; i += blockDim.x) {
+        const int j = i / nb, k = i - j * nb;
+        const double* row = D.grid + (size_t)j * nb;
+        const double* row_lo = D.grid + (size_t)d * nb + (size_t)j * nb;
+        slot_cell(D, j, k, edge_left(row, row_lo, k), edge_right(row, row_lo, k), inv_g);
+    }
     if (threadIdx.x == 0) {
         BatchState z;
         memset(&z, 0, sizeof z);
@@ -469,7 +490,7 @@ void BatchEngine::partition(const std::vector<int>& live, int* nseg_out)
                     g.adjust = adjust ? 1u : 0u;
                     g.c0 = c;
                     g.c1 = cend;
-                    g.perm_k = cube_permutation(cend - c);
+                    set_cube_order(g, cend - c);
                     g.hist_off = hist_off;
                     if (adjust) hist_off += (size_t)hdesc_[s].d * hdesc_[s].nb;
                     c = cend;

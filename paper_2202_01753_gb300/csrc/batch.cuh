@@ -57,8 +57,8 @@ vsample_batch_kernel(const __grid_constant__ BatchArgs a)
         const uint32_t nb = sd.nb;
         Cell* cells = reinterpret_cast<Cell*>(smem);
         HT* hist = reinterpret_cast<HT*>(smem + cell_bytes(MIXED) * d * nb);
-        if (adjust) stage_cells<MIXED, true>(cells, hist, sd.cells, d, nb, d);
-        else stage_cells<MIXED, false>(cells, hist, sd.cells, d, nb, d);
+        if (adjust) clear_hist(hist, d * nb);
+        stage_cells<MIXED>(cells, sd.cells, d, nb);
         __syncthreads();
 
         const BatchView v{d,        nb,           sd.g,     sd.gmagic,         sd.key0,          sd.key1, d,
@@ -68,7 +68,7 @@ vsample_batch_kernel(const __grid_constant__ BatchArgs a)
         CubeSums acc;
         auto sample = [&](auto adj_c, auto fix_c) {
             sample_cubes<FAM, MIXED, decltype(adj_c)::value, NB4, D, decltype(fix_c)::value>(
-                v, cells, hist, seg.c0, seg.c1 - seg.c0, seg.perm_k, 0, 1, it, sd.lanes, sd.p, acc);
+                v, cells, hist, seg.c0, seg.c1 - seg.c0, seg.perm_k, seg.perm_inv, 0, 1, it, sd.lanes, sd.p, acc);
         };
         bool done = false;
         if constexpr (!MIXED && FixFamily<FAM>::kHas) {
@@ -82,7 +82,7 @@ vsample_batch_kernel(const __grid_constant__ BatchArgs a)
             if (adjust) sample(std::true_type{}, std::false_type{});
             else sample(std::false_type{}, std::false_type{});
         }
-        block_write_sums(acc, red, a.seg_part + 3 * (size_t)si);
+        block_write_sums<MIXED>(acc, false, red, a.seg_part + 3 * (size_t)si);
         if (adjust) {
             __syncthreads();
             HT* out = reinterpret_cast<HT*>(a.seg_hist) + seg.hist_off;

@@ -564,7 +564,14 @@ mcubes_status mcubes_setup(mcubes_ctx* c, int id, const double* params, int npar
         c->split = (int)std::max(1LL, std::min(want, p / threads));
         if (c->split > 1) c->grid_adj = c->grid_noadj = (int)(m * c->split);
     }
-    const int grid_max = std::max(c->grid_adj, c->grid_noadj);
+    // no more blocks than the cubes fill (each one stages the grid, flushes its
+    // histogram and adds a partial to the refinement's sums)
+    if (c->split == 1) {
+        const int fill = (int)std::min<long long>((m * c->lanes + threads - 1) / threads, INT32_MAX);
+        c->grid_adj = std::min(c->grid_adj, fill);
+        c->grid_noadj = std::min(c->grid_noadj, fill);
+    }
+    const int grid_max = std::max(std::max(c->grid_adj, c->grid_noadj), std::max(c->grid_res_adj, c->grid_res_noadj));
 
     // device buffers
     MC_CHECK(c, c->grid.reserve(2 * sizeof(double) * d * nb));  // high parts, then low parts
@@ -592,7 +599,7 @@ mcubes_status mcubes_setup(mcubes_ctx* c, int id, const double* params, int npar
     a.split = (uint32_t)c->split;
     a.cube_begin = 0;
     a.cube_end = (uint64_t)m;
-    a.perm_k = cube_permutation((uint64_t)m);
+    set_cube_order(a, (uint64_t)m);
     philox_round_keys(c->opts.seed, a.rk);
     for (int j = 0; j < d; ++j) {
         a.lo[j] = lo[j];
@@ -614,7 +621,7 @@ mcubes_status mcubes_setup(mcubes_ctx* c, int id, const double* params, int npar
     r.part = (const double*)c->part.ptr;
     r.hist_acc = (double*)c->hist_acc.ptr;
     r.cells_g = c->cells.ptr;
-    r.g = (uint32_t)g;
+    r.inv_g = 1.0 / (double)g;
     r.mixed = c->mixed ? 1 : 0;
     std::memset(&c->cellbox, 0, sizeof c->cellbox);
     for (int j = 0; j < d; ++j) {
@@ -798,7 +805,7 @@ mcubes_status mcubes_sample_range(mcubes_ctx* c, unsigned it, int adjust, long l
     a.want_abs = 1;  // the pass reports the sum of |cube mean|
     a.cube_begin = (uint64_t)cube_begin;
     a.cube_end = (uint64_t)cube_end;
-    a.perm_k = cube_permutation((uint64_t)(cube_end - cube_begin));
+    set_cube_order(a, (uint64_t)(cube_end - cube_begin));
     const bool adj = adjust != 0;
     const int grid = adj ? c->grid_adj : c->grid_noadj;
     const size_t smem = adj ? c->smem_adj : c->smem_noadj;
@@ -839,7 +846,7 @@ mcubes_status mcubes_shard_sample(mcubes_ctx* c, long long cube_begin, long long
     a.split = 1;  // a range pass: the partials are sums over whole cubes
     a.cube_begin = (uint64_t)cube_begin;
     a.cube_end = (uint64_t)cube_end;
-    a.perm_k = cube_permutation((uint64_t)(cube_end - cube_begin));
+    set_cube_order(a, (uint64_t)(cube_end - cube_begin));
     const int grid = adjust ? c->grid_res_adj : c->grid_res_noadj;
     const size_t smem = adjust ? c->smem_adj : c->smem_noadj;
     EventPair ev;

@@ -87,12 +87,9 @@ __device__ __forceinline__ LogPair ld_pair(const LogPair* p)
 // the table point at or below m, r = (m - c_j)/c_j in [0, 2^-8), d_k =
 // 1 + k/65536 the second table point at or below 1 + r and r2 = (r - k/65536)/d_k
 // in [0, 2^-16): every quantity is non-negative.
-__device__ __forceinline__ double fx_log(double x)
+// The mantissa's part, from its 52 fraction bits f: ln m in Q64 (< ln 2).
+__device__ __forceinline__ uint64_t fx_ln_mantissa(uint64_t f)
 {
-    const uint64_t u = (uint64_t)__double_as_longlong(x);
-    if ((uint32_t)(u >> 32) - 0x00100000u >= 0x7FE00000u) return log_slow(x);  // not a positive normal number
-    const int e = (int)(u >> 52) - 1023;
-    const uint64_t f = u & 0xFFFFFFFFFFFFFull;
     const int j = (int)(f >> 44);
     // m - c_j is the mantissa's low 44 bits (Q52); r = (m - c_j)/c_j in Q64 (< 2^56)
     const LogPair cj = ld_pair(&kLogC[j]);
@@ -109,7 +106,16 @@ __device__ __forceinline__ double fx_log(double x)
     const uint64_t sq = ((uint64_t)H * H) >> 32;                           // r2^2, Q64 (< 2^32)
     const uint32_t cube = (uint32_t)(((uint64_t)(uint32_t)sq * H) >> 48);  // r2^3, Q64 (< 2^16)
     const uint64_t l2 = R - (sq >> 1) + __umulhi(cube, q32_inv(3));        // ln(1 + r2), Q64
-    const uint64_t U = cj.ln + dk.ln + l2;                                 // ln m, Q64 (< ln 2)
+    return cj.ln + dk.ln + l2;
+}
+
+__device__ __forceinline__ double fx_log(double x)
+{
+    const uint64_t u = (uint64_t)__double_as_longlong(x);
+    if ((uint32_t)(u >> 32) - 0x00100000u >= 0x7FE00000u) return log_slow(x);  // not a positive normal number
+    const int e = (int)(u >> 52) - 1023;
+    const uint64_t f = u & 0xFFFFFFFFFFFFFull;
+    const uint64_t U = fx_ln_mantissa(f);  // ln m, Q64 (< ln 2)
     // e ln 2 + ln m as sign and 128-bit magnitude in Q64; |e| < 2^11, so
     // |e| ln 2 is two 32 x 32-bit products (ln 2 = L1 2^32 + L0)
     const uint32_t ae = (uint32_t)(e < 0 ? -e : e);
@@ -316,6 +322,32 @@ __device__ __forceinline__ uint64_t fx_recip(uint64_t m)
     const uint64_t e1 = (1ull << 63) - __umul64hi(m, y1);                       // Q63 (< 2^24)
     const uint64_t y2 = y1 + (((y1 >> 32) * (uint64_t)(uint32_t)e1) >> 31);
     return y2 < (1ull << 63) ? (1ull << 63) : y2;  // x next to 2: the truncations may fall short of 1/2
+}
+
+__device__ __forceinline__ float rsqrt_seed(float x)
+{
+#ifdef __CUDA_ARCH__
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+#else
+    return 1.0f / std::sqrt(x);
+#endif
+}
+
+// sqrt(M 2^-64) as Q63 for M in [2^62, 2^64): s = M y from a single-precision
+// seed y of the reciprocal root, then two steps s + (M - s^2) y / 2 (Newton's
+// with y kept) in fixed point: relative error below 2^-58.
+__device__ __forceinline__ uint64_t fx_sqrt(uint64_t M)
+{
+    const float xf = (float)(uint32_t)(M >> 40) * 5.9604644775390625e-08f;  // in [1/4, 1)
+    const int64_t y = (int64_t)(uint32_t)fminf(rsqrt_seed(xf) * 2147483648.0f, 4294967040.0f);  // Q31
+    uint64_t s = (M >> 32) * (uint64_t)y;                                   // Q63
+    int64_t dl = (int64_t)((M >> 2) - __umul64hi(s, s));                    // M - s^2, Q62 (below 2^42)
+    s += (uint64_t)(((dl >> 10) * y) >> 21);
+    dl = (int64_t)((M >> 2) - __umul64hi(s, s));
+    s += (uint64_t)((dl * y) >> 31);
+    return s;
 }
 
 // cos(2 pi t) for the fraction of a turn t = a 2^-64: sign and magnitude, the

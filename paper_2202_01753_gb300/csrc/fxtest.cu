@@ -37,10 +37,17 @@ __device__ int g_rebin_flags[2];  // error, done
 __global__ void __launch_bounds__(mc::kRefineThreads)
 rebin_kernel(int nb, double alpha, double* C, double* B, double* Blo)
 {
-    __shared__ double scratch[33];
-    // the histogram is its own single partial; its sum is written back in place
-    mc::refine_detail::rebin_axis(C, 0, 1, false, nb, alpha, B, Blo, C, &g_rebin_flags[0], &g_rebin_flags[1],
-                                  scratch);
+    __shared__ mc::refine_detail::RebinShared s;
+    for (int k = threadIdx.x; k < nb; k += mc::kRefineThreads) {
+        s.C[k] = C[k];
+        s.B[k] = B[k];
+        s.Blo[k] = Blo[k];
+    }
+    if (!mc::refine_detail::rebin_block(s, nb, alpha, &g_rebin_flags[0], &g_rebin_flags[1])) return;
+    for (int k = threadIdx.x; k < nb; k += mc::kRefineThreads) {
+        B[k] = s.B[k];
+        Blo[k] = s.Blo[k];
+    }
 }
 
 }  // namespace

@@ -10,42 +10,21 @@
 
 namespace mc {
 
+// Programmatic dependent launch (launch_dependent): a kernel's blocks may be
+// placed, and run up to their wait, once every block of the kernel before it
+// in the stream has called grid_dependents_launch or ended; the wait ends when
+// that kernel has completed and its writes are visible.
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---------------------------------------------------------------------------
-// Double-double arithmetic (value = hi + lo, |lo| <= ulp(hi)/2): error-free
-// TwoSum (Knuth) and an FMA-based exact product (Dekker).  Grid edges are held
-// in this form so that a narrow bin's width (a difference of two nearly equal
-// edges, and a factor of the Jacobian) keeps full relative precision; the
-// rebinning forms each new edge (left + width * fraction) in it.
+// Double-double numbers (value = hi + lo, |lo| <= ulp(hi)/2).  Grid edges are
+// held in this form so that a narrow bin's width (a difference of two nearly
+// equal edges, and a factor of the Jacobian) keeps full relative precision.
 // ---------------------------------------------------------------------------
 struct DD {
     double hi, lo;
 };
-
-__device__ __forceinline__ DD dd_two_sum(double a, double b)
-{
-    const double s = __dadd_rn(a, b);
-    const double bb = __dsub_rn(s, a);
-    return DD{s, __dadd_rn(__dsub_rn(a, __dsub_rn(s, bb)), __dsub_rn(b, bb))};
-}
-
-__device__ __forceinline__ DD dd_renorm(double hi, double lo)
-{
-    const double s = __dadd_rn(hi, lo);
-    return DD{s, __dsub_rn(lo, __dsub_rn(s, hi))};
-}
-
-__device__ __forceinline__ DD dd_add(DD a, DD b)
-{
-    const DD t = dd_two_sum(a.hi, b.hi);
-    return dd_renorm(t.hi, __dadd_rn(__dadd_rn(t.lo, a.lo), b.lo));
-}
-
-__device__ __forceinline__ DD dd_scale(DD a, double b)
-{
-    const double p = __dmul_rn(a.hi, b);
-    const double e = __fma_rn(a.hi, b, -p);
-    return dd_renorm(p, __fma_rn(a.lo, b, e));
-}
 
 // ---------------------------------------------------------------------------
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, "Parallel random numbers: as easy
@@ -156,47 +135,107 @@ __device__ __forceinline__ double int_prod_value(const IntProd& p)
 }
 
 // ---------------------------------------------------------------------------
-// Map cell k of one axis in the box's coordinates, from the double-double
-// right edges (unit cube) of that axis's row: (x left edge, x width / g) for
-// the FP64 kernels, (x left edge, nb * x width) in single precision for the
-// mixed ones.  inv_g = 1 / g.
+// Grid edges as 128-bit integers.  The edges are kept in double-double (see
+// above); the rebinning and the cells take differences and fractions of them
+// in integers scaled by the right edge's exponent E (v -> v 2^(126 - E), so
+// the right edge fills the word), where a dependent operation takes a few
+// cycles against 66 for an FP64 one.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void map_cell_edges(DD left, DD right, double lo, double scale, double* xl, double* xw)
+using u128 = unsigned __int128;
+
+__device__ __forceinline__ int clz_u128(u128 v)  // v > 0
 {
-    const DD wd = dd_add(right, DD{-left.hi, -left.lo});
-    *xl = lo + scale * left.hi;
-    *xw = scale * (wd.hi + wd.lo);
+    const uint64_t hi = (uint64_t)(v >> 64);
+    return hi ? __clzll((long long)hi) : 64 + __clzll((long long)(uint64_t)v);
 }
 
-__device__ __forceinline__ void map_cell(const double* row, const double* row_lo, uint32_t k, double lo,
-                                         double scale, double* xl, double* xw)
+__device__ __forceinline__ int exponent_of(double v) { return (int)(((uint64_t)__double_as_longlong(v) >> 52) & 0x7FF) - 1023; }
+
+// |v| 2^(126 - E), |v| < 2^(E + 1)
+__device__ __forceinline__ u128 scaled_u128(double v, int E)
 {
-    const DD right{row[k], row_lo[k]};
-    const DD left = k ? DD{row[k - 1], row_lo[k - 1]} : DD{0.0, 0.0};
-    map_cell_edges(left, right, lo, scale, xl, xw);
+    const uint64_t b = (uint64_t)__double_as_longlong(v);
+    const int e = (int)((b >> 52) & 0x7FF);
+    const uint64_t mant = (b & 0xFFFFFFFFFFFFFull) | (e ? 1ull << 52 : 0ull);
+    const int sh = 74 - (E - ((e ? e : 1) - 1023));
+    if (sh >= 0) return (u128)mant << sh;
+    return sh > -64 ? (u128)(mant >> -sh) : (u128)0;
 }
 
-__device__ __forceinline__ double2 map_cell_f64(const double* row, const double* row_lo, uint32_t k, double lo,
-                                                double scale, double inv_g)
+__device__ __forceinline__ u128 edge_u128(DD v, int E)
 {
-    double xl, xw;
-    map_cell(row, row_lo, k, lo, scale, &xl, &xw);
-    return make_double2(xl, xw * inv_g);
+    const u128 h = scaled_u128(v.hi, E), l = scaled_u128(v.lo, E);
+    return __double_as_longlong(v.lo) < 0 ? h - l : h + l;
+}
+
+// v 2^(E - 126) as a double-double: the high part rounded to 53 bits, the
+// rest (of either sign) to 53 more; v > 0, v < 2^127
+__device__ __forceinline__ DD edge_from_u128(u128 v, int E)
+{
+    const int z = clz_u128(v);
+    const u128 n = v << z;
+    const uint64_t mant = ((uint64_t)(n >> 75)) + ((uint64_t)(n >> 74) & 1ull);  // 2^52..2^53
+    const uint64_t hb = ((uint64_t)(E - z + 1024) << 52) + (mant - (1ull << 52));
+    const u128 back = (u128)mant << 75;  // 0 stands for 2^128 after a carry: the difference wraps right
+    const bool neg = ((uint64_t)(n >> 74) & 1ull) != 0;
+    const u128 mag = neg ? back - n : n - back;  // <= 2^74
+    uint64_t lb = 0;
+    if (mag != 0) {
+        const int y = clz_u128(mag);
+        const uint64_t m = (uint64_t)((mag << y) >> 75);  // 53 bits
+        const int be = E + 1 - y - z + 1023;
+        if (be >= 1) lb = ((uint64_t)neg << 63) | (((uint64_t)be << 52) + (m - (1ull << 52)));
+    }
+    return DD{__longlong_as_double((long long)hb), __longlong_as_double((long long)lb)};
+}
+
+// right - left > 0 as a 64-bit significand and exponent (m = 0: no width)
+__device__ __forceinline__ IntProd edge_width(DD left, DD right)
+{
+    const int E = exponent_of(right.hi);
+    const u128 w = edge_u128(right, E) - edge_u128(left, E);
+    if (w == 0) return IntProd{0ull, 0};
+    const int z = clz_u128(w);
+    return IntProd{(uint64_t)((w << z) >> 64), E + 1 - z};
+}
+
+// ---------------------------------------------------------------------------
+// Map cell of one axis in the box's coordinates, from the double-double edges
+// (unit cube) at its two sides: (x left edge, x width / g) for the FP64
+// kernels, (x left edge, nb * x width) in single precision for the mixed
+// ones.  inv_g = 1 / g.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ double2 map_cell_f64(DD left, DD right, double lo, double scale, double inv_g)
+{
+    const IntProd w = edge_width(left, right);
+    const double wd = w.m ? int_prod_value(w) : 0.0;
+    return make_double2(lo + scale * left.hi, scale * wd * inv_g);
 }
 
 // Map cell of the fixed-point form: (t at the left edge as an integer with
-// m.fbits fraction bits, t width / g as a double).
-__device__ __forceinline__ double2 map_cell_fix(DD left, DD right, const CellMap& m, int j, double inv_g)
+// m.fbits fraction bits, t width / g as a double), in integers but for none.
+__device__ __forceinline__ double2 map_cell_fix(DD left, DD right, const CellMap& m, int j)
 {
-    const DD wd = dd_add(right, DD{-left.hi, -left.lo});
-    const double w = (m.b[j] * (wd.hi + wd.lo)) * inv_g;
-    // b left in two parts, each converted to an integer by itself: short
-    // dependent chains (a dependent FP64 instruction takes 66 cycles)
-    const double sc = __longlong_as_double((long long)(1023 + m.fbits) << 52);  // 2^fbits
-    const double p = __dmul_rn(m.b[j], left.hi);
-    const double e = fma(m.b[j], left.lo, fma(m.b_lo[j], left.hi, __fma_rn(m.b[j], left.hi, -p)));
-    const long long L = m.a[j] + __double2ll_rn(p * sc) + __double2ll_rn(e * sc);
-    return make_double2(__longlong_as_double(L), w);
+    const int E = exponent_of(right.hi);
+    const u128 lu = edge_u128(left, E);
+    const u128 w = edge_u128(right, E) - lu;
+    double width = 0.0;
+    if (w != 0) {
+        const int z = clz_u128(w);
+        width = int_prod_value(int_prod_mul2(IntProd{(uint64_t)((w << z) >> 64), E + 1 - z},
+                                             IntProd{m.bg_m[j], m.bg_e[j]}));
+    }
+    const int sh = 62 - E;  // the left edge (< 1) as Q64
+    const uint64_t l64 = sh < 128 ? (uint64_t)(lu >> sh) : 0ull;
+    return make_double2(__longlong_as_double(m.a[j] + (long long)__umul64hi(m.b[j], l64)), width);
+}
+
+__device__ __forceinline__ float2 map_cell_f32(DD left, DD right, double lo, double scale, uint32_t nb)
+{
+    const IntProd w = edge_width(left, right);
+    const double wd = w.m ? int_prod_value(w) : 0.0;
+    const double xl = lo + scale * left.hi, xw = scale * wd;
+    return make_float2((float)xl, (float)(xw * (double)nb));
 }
 
 __device__ __forceinline__ DD edge_right(const double* row, const double* row_lo, uint32_t k)
@@ -207,14 +246,6 @@ __device__ __forceinline__ DD edge_right(const double* row, const double* row_lo
 __device__ __forceinline__ DD edge_left(const double* row, const double* row_lo, uint32_t k)
 {
     return k ? DD{row[k - 1], row_lo[k - 1]} : DD{0.0, 0.0};
-}
-
-__device__ __forceinline__ float2 map_cell_f32(const double* row, const double* row_lo, uint32_t k, double lo,
-                                               double scale, uint32_t nb)
-{
-    double xl, xw;
-    map_cell(row, row_lo, k, lo, scale, &xl, &xw);
-    return make_float2((float)xl, (float)(xw * (double)nb));
 }
 
 // ---------------------------------------------------------------------------

@@ -43,7 +43,7 @@ __host__ __device__ constexpr size_t hist_bytes(bool mixed) { return mixed ? 4 :
 // host.  One instance per single-integral context.
 struct DevState {
     uint32_t it;        // iteration index of the next sampling pass
-    int done;           // converged or failed: further iterations are skipped
+    int done;           // converged or failed: further iterations are skipped (read with it, 8 bytes)
     int active;         // set by the sampling launch: this iteration ran
     int error;          // mcubes_status of a failure seen on the device
     int n;              // iterations recorded
@@ -86,12 +86,13 @@ struct FamParams {
 };
 
 // Cells of the fixed-point form: coordinate t = a + b x (x the unit-cube edge)
-// with fbits fraction bits (0: cells in the box's coordinates); b is a
-// double-double.  Sums wrap around 2^64 (OSC: t in turns, whole ones do not
-// matter).
+// with fbits fraction bits (0: cells in the box's coordinates); a, b as such
+// integers, b / g as bg_m 2^(bg_e - 63).  Sums wrap around 2^64 (OSC: t in
+// turns, whole ones do not matter).
 struct CellMap {
     long long a[kDMax];
-    double b[kDMax], b_lo[kDMax];
+    uint64_t b[kDMax], bg_m[kDMax];
+    int bg_e[kDMax];
     int fbits, pad;
 };
 
@@ -115,6 +116,7 @@ struct VsArgs {
                                 // each block's shifted sums (K, S1, S2) of its slice of one cube)
     uint64_t cube_begin, cube_end;
     uint64_t perm_k;          // cube order: logical i -> cube_begin + (i perm_k mod n), gcd(perm_k, n) = 1
+    uint64_t perm_inv;        // floor((2^64 - 1) / n) (set_cube_order sets both)
     uint32_t rk[10][2];       // Philox round keys (key + r * Weyl constants)
     double lo[kDMax];
     double scale[kDMax];      // hi - lo
@@ -170,7 +172,7 @@ struct BatchSeg {
     uint32_t adjust;            // host: adjusting at the step's first iteration (the histogram space is
                                 // reserved); device: whether this iteration adjusts
     uint64_t c0, c1;
-    uint64_t perm_k;            // cube order within the segment (see sample_cubes)
+    uint64_t perm_k, perm_inv;  // cube order within the segment (see sample_cubes)
     uint64_t hist_off;          // element offset of the segment's partial histogram
 };
 
@@ -215,7 +217,7 @@ struct RefineArgs {
     void* cells_g;            // [d][nb] map cells, rebuilt for every rebinned axis (null: none kept)
     double lo[kDMax], scale[kDMax];
     CellMap cm;               // cm.fbits > 0: cells of the fixed-point form
-    uint32_t g;
+    double inv_g;             // 1 / g
     int mixed;
     DevState* st;
     int nblocks, d, nb, adjust;
@@ -236,6 +238,27 @@ struct CellBox {
 cudaError_t launch_cells(const double* grid, const double* grid_lo, const CellBox& box, int d, int nb, void* out,
                          cudaStream_t s);
 
+// Launches a kernel that waits for its predecessor itself (every thread calls
+// grid_dependency_wait before it touches memory the predecessor writes, also
+// when it has nothing to do, so that "complete" stays transitive along the
+// stream): its launch and set-up overlap the predecessor's end.  On the
+// legacy default stream, a plain launch.
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*k)(P...), int grid, int threads, size_t smem, cudaStream_t s, const A&... args)
+{
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3((unsigned)grid);
+    c.blockDim = dim3((unsigned)threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = s ? 1 : 0;
+    return cudaLaunchKernelEx(&c, k, args...);
+}
+
 // Launchers (one per integrand family translation unit).
 cudaError_t launch_vsample(int family, bool mixed, bool adjust, const VsArgs& a, int grid,
                            size_t smem, cudaStream_t s);
@@ -248,6 +271,11 @@ cudaError_t vsample_occupancy(int family, bool mixed, bool adjust, bool fix, int
 void affine_prepare(int id, const double* params, int d, const double* lo, const double* scale, long long g, int nb,
                     FamParams* fp, CellMap* cm, double* jac0);
 uint64_t cube_permutation(uint64_t n);
+template <class T> void set_cube_order(T& a, uint64_t n)  // of a range of n cubes
+{
+    a.perm_k = cube_permutation(n);
+    a.perm_inv = n ? ~0ull / n : 0ull;
+}
 // Raises a kernel's dynamic shared-memory limit on the current device to at
 // least smem bytes (never lowers it, so that contexts of different sizes can
 // share a kernel); a host-side record skips the driver call when the limit

@@ -139,7 +139,7 @@ extern "C" mcubes_status mcubes_sample_range_noalloc(
         a.split = 1;
         a.cube_begin = (uint64_t)cube_begin;
         a.cube_end = (uint64_t)cube_end;
-        a.perm_k = cube_permutation((uint64_t)(cube_end - cube_begin));
+        set_cube_order(a, (uint64_t)(cube_end - cube_begin));
         philox_round_keys(seed, a.rk);
         for (int j = 0; j < d; ++j) {
             a.lo[j] = lo[j];

@@ -129,37 +129,38 @@ template <> struct Prec<true> {
     using S = std::conditional_t<MC_MIXED_CUBE_F64 != 0, double, float>;
 };
 
-// Stages the grid of all axes into shared-memory cells and clears the
-// histogram ([hist_d][nb]).  grid/grid_lo: [d][nb] double-double right
+// Clears a block's histogram ([hist_d][nb]).
+template <class HT>
+__device__ __forceinline__ void clear_hist(HT* hist, uint32_t n)
+{
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) hist[i] = HT(0);
+}
+
+// Stages the grid of all axes into shared-memory cells.  grid/grid_lo: [d][nb] double-double right
 // edges (unit cube); lo/scale: the box's lower corner and hi - lo; g:
 // sub-cubes per axis.
-template <bool MIXED, bool ADJ, bool FIX, class Arr>
-__device__ __forceinline__ void stage_grid(typename Prec<MIXED>::Cell* cells, typename Prec<MIXED>::H* hist,
-                                           const double* grid, const double* grid_lo, const Arr& lo,
-                                           const Arr& scale, const CellMap& cm, uint32_t d, uint32_t nb, uint32_t g,
-                                           uint32_t hist_d)
+template <bool MIXED, bool FIX, class Arr>
+__device__ __forceinline__ void stage_grid(typename Prec<MIXED>::Cell* cells, const double* grid,
+                                           const double* grid_lo, const Arr& lo, const Arr& scale, const CellMap& cm,
+                                           uint32_t d, uint32_t nb, uint32_t g)
 {
-    if constexpr (ADJ)
-        for (uint32_t i = threadIdx.x; i < hist_d * nb; i += blockDim.x) hist[i] = typename Prec<MIXED>::H(0);
     const double inv_g = 1.0 / (double)g;  // one division per thread, a multiply per cell
     for (uint32_t i = threadIdx.x; i < d * nb; i += blockDim.x) {
         const uint32_t j = i / nb, k = i - j * nb;
-        if constexpr (MIXED) cells[i] = map_cell_f32(grid + j * nb, grid_lo + j * nb, k, lo[j], scale[j], nb);
-        else if constexpr (FIX)
-            cells[i] = map_cell_fix(edge_left(grid + j * nb, grid_lo + j * nb, k),
-                                    edge_right(grid + j * nb, grid_lo + j * nb, k), cm, (int)j, inv_g);
-        else cells[i] = map_cell_f64(grid + j * nb, grid_lo + j * nb, k, lo[j], scale[j], inv_g);
+        const DD left = edge_left(grid + j * nb, grid_lo + j * nb, k);
+        const DD right = edge_right(grid + j * nb, grid_lo + j * nb, k);
+        if constexpr (MIXED) cells[i] = map_cell_f32(left, right, lo[j], scale[j], nb);
+        else if constexpr (FIX) cells[i] = map_cell_fix(left, right, cm, (int)j);
+        else cells[i] = map_cell_f64(left, right, lo[j], scale[j], inv_g);
     }
 }
 
 // The same staging from cells already built in global memory (by the
 // refinement after each rebin, and at set-up): a copy, 16-byte words.
-template <bool MIXED, bool ADJ>
-__device__ __forceinline__ void stage_cells(typename Prec<MIXED>::Cell* cells, typename Prec<MIXED>::H* hist,
-                                            const void* cells_g, uint32_t d, uint32_t nb, uint32_t hist_d)
+template <bool MIXED>
+__device__ __forceinline__ void stage_cells(typename Prec<MIXED>::Cell* cells, const void* cells_g, uint32_t d,
+                                            uint32_t nb)
 {
-    if constexpr (ADJ)
-        for (uint32_t i = threadIdx.x; i < hist_d * nb; i += blockDim.x) hist[i] = typename Prec<MIXED>::H(0);
     const uint32_t bytes = d * nb * (uint32_t)sizeof(typename Prec<MIXED>::Cell);
     const uint4* src = static_cast<const uint4*>(cells_g);
     uint4* dst = reinterpret_cast<uint4*>(cells);
@@ -357,6 +358,17 @@ struct CubeSums {
     __device__ double vA() const { return A + fA.value(); }
 };
 
+// x mod n with inv = floor((2^64 - 1)/n) from the host (a 64-bit division is
+// ~100 dependent instructions, most of a small launch's set-up); n = 0: 0.
+__device__ __forceinline__ uint64_t mod_by(uint64_t x, uint64_t n, uint64_t inv)
+{
+    if (n == 0) return 0;
+    uint64_t r = x - __umul64hi(x, inv) * n;  // the quotient is short by 2 at most
+    if (r >= n) r -= n;
+    if (r >= n) r -= n;
+    return r;
+}
+
 // Samples cubes [cube_lo, cube_lo + ncubes) of one integral.  The block takes
 // groups of (blockDim / lanes) logical cube indices: group0, group0 + gstride,
 // ...; logical index i is cube cube_lo + (i * perm_k mod ncubes), a bijection
@@ -370,8 +382,8 @@ struct CubeSums {
 template <int FAM, bool MIXED, bool ADJ, int NB4, int DC, bool FIX, class A>
 __device__ __forceinline__ void sample_cubes(const A& a, const typename Prec<MIXED>::Cell* cells,
                                              typename Prec<MIXED>::H* hist, uint64_t cube_lo, uint64_t ncubes,
-                                             uint64_t perm_k, uint64_t group0, uint64_t gstride, uint32_t it,
-                                             uint32_t lanes, uint32_t p, CubeSums& acc)
+                                             uint64_t perm_k, uint64_t perm_inv, uint64_t group0, uint64_t gstride,
+                                             uint32_t it, uint32_t lanes, uint32_t p, CubeSums& acc)
 {
     using R = typename Prec<MIXED>::R;
     using HT = typename Prec<MIXED>::H;
@@ -394,14 +406,16 @@ __device__ __forceinline__ void sample_cubes(const A& a, const typename Prec<MIX
         inv_var_den = a.inv_var_den;
     }
     const uint64_t first = group0 * cubes_per_group + threadIdx.x / L;
-    uint64_t off = ncubes ? (first % ncubes) * perm_k % ncubes : 0;               // physical offset of `first`
-    const uint64_t step = ncubes ? (gstride * cubes_per_group % ncubes) * perm_k % ncubes : 0;
+    // physical offset of `first`, and its step from group to group (below 2^32, as the cube counter)
+    uint32_t off = (uint32_t)mod_by(mod_by(first, ncubes, perm_inv) * perm_k, ncubes, perm_inv);
+    const uint32_t step =
+        (uint32_t)mod_by(mod_by(gstride * cubes_per_group, ncubes, perm_inv) * perm_k, ncubes, perm_inv);
     for (uint64_t base = group0 * cubes_per_group; base < ncubes; base += gstride * cubes_per_group) {
         const uint64_t ci = base + threadIdx.x / L;
         const bool valid = ci < ncubes;
-        const uint32_t c = (uint32_t)(cube_lo + (valid ? off : 0));
+        const uint32_t c = (uint32_t)cube_lo + (valid ? off : 0u);
         off += step;
-        if (off >= ncubes) off -= ncubes;
+        if (off < step || off >= (uint32_t)ncubes) off -= (uint32_t)ncubes;
         // sub-cube digits (axis 0 fastest), kept as nb * digit
         uint32_t nbc[DN];
         {
@@ -585,34 +599,43 @@ __device__ __forceinline__ void sample_cube_slice(const A& a, const typename Pre
     }
 }
 
-// Fixed-order block sum of the three per-thread sums; thread 0 writes them.
-template <int NW>
-__device__ __forceinline__ void block_write_sums(const CubeSums& acc, double (*red)[NW], double* out)
+// Fixed-order block sum of the per-thread sums; out[2] (the sum of |cube
+// mean|) only where it is wanted.  A block's FP64 additions take the SM's
+// pipe 16 cycles each whatever the number of active lanes, and 32 resident
+// warps with three five-step shuffle trees spent ~8000 cycles here: lanes
+// 0-15 and 16-31 first swap halves and then sum one quantity each, five
+// additions for both, and the warps' sums are added the same way.
+template <bool MIXED, int NW>
+__device__ __forceinline__ void block_write_sums(const CubeSums& acc, bool want_abs, double (*red)[NW], double* out)
 {
-    double v0 = acc.vI(), v1 = acc.vV(), v2 = acc.vA();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool up = lane >= 16;
+    const double vI = MIXED ? acc.vI() : acc.I, vV = MIXED ? acc.vV() : acc.V;
+    double v = (up ? vV : vI) + __shfl_xor_sync(0xffffffffu, up ? vI : vV, 16);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        v0 += __shfl_down_sync(0xffffffffu, v0, off);
-        v1 += __shfl_down_sync(0xffffffffu, v1, off);
-        v2 += __shfl_down_sync(0xffffffffu, v2, off);
-    }
-    const int warp = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) {
-        red[0][warp] = v0;
-        red[1][warp] = v1;
-        red[2][warp] = v2;
+    for (int off = 8; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    if ((lane & 15) == 0) red[up][warp] = v;
+    if (want_abs) {
+        double a = MIXED ? acc.vA() : acc.A;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+        if (lane == 0) red[2][warp] = a;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            s0 += red[0][w];
-            s1 += red[1][w];
-            s2 += red[2][w];
-        }
-        out[0] = s0;
-        out[1] = s1;
-        out[2] = s2;
+    if (warp != 0) return;
+    if (!want_abs && lane == 0) out[2] = 0.0;
+    const int nw = (int)(blockDim.x >> 5);
+    const int w = lane & 15;
+    v = w < nw ? red[up][w] : 0.0;
+    if (nw > 16 && w + 16 < nw) v += red[up][w + 16];
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    if ((lane & 15) == 0) out[up] = v;
+    if (want_abs) {
+        double a = lane < nw ? red[2][lane] : 0.0;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+        if (lane == 0) out[2] = a;
     }
 }
 
@@ -637,6 +660,13 @@ constexpr int vsample_kernel_min_blocks()
                                                         : 1024 / vsample_threads(FAM, MIXED, D);
 }
 
+__device__ __forceinline__ int2 ld_volatile_int2(const void* p)
+{
+    int2 v;
+    asm volatile("ld.volatile.global.v2.s32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+    return v;
+}
+
 // One instantiation per dimension D: with the axis count a compile-time
 // constant every per-axis loop is unrolled without guards and the families'
 // dimension-dependent code (the corner family's power) folds (corner8: 21.4
@@ -656,18 +686,22 @@ vsample_kernel(const __grid_constant__ VsArgs a)
 
     constexpr uint32_t d = D;
     const uint32_t nb = a.nb;
-    uint32_t it = a.it_fixed;
-    if (a.st != nullptr) {
-        const int done = *(volatile const int*)&a.st->done;
-        if (blockIdx.x == 0 && threadIdx.x == 0) a.st->active = done ? 0 : 1;
-        if (done) return;
-        it = *(volatile const uint32_t*)&a.st->it;
-    }
-
     Cell* cells = reinterpret_cast<Cell*>(smem);
     HT* hist = reinterpret_cast<HT*>(smem + cell_bytes(MIXED) * d * nb);
-    if (a.cells_g) stage_cells<MIXED, ADJ>(cells, hist, a.cells_g, d, nb, a.hist_d);
-    else stage_grid<MIXED, ADJ, FIX>(cells, hist, a.grid, a.grid_lo, a.lo, a.scale, a.cm, d, nb, a.g, a.hist_d);
+    if constexpr (ADJ) clear_hist(hist, a.hist_d * nb);
+    grid_dependency_wait();  // the refinement before this pass (launch_dependent)
+    uint32_t it = a.it_fixed;
+    if (a.st != nullptr) {
+        // iteration index and flag by one load
+        const int2 v = ld_volatile_int2(&a.st->it);
+        const int done = v.y;
+        if (blockIdx.x == 0 && threadIdx.x == 0) a.st->active = done ? 0 : 1;
+        if (done) return;
+        it = (uint32_t)v.x;
+    }
+
+    if (a.cells_g) stage_cells<MIXED>(cells, a.cells_g, d, nb);
+    else stage_grid<MIXED, FIX>(cells, a.grid, a.grid_lo, a.lo, a.scale, a.cm, d, nb, a.g);
     __syncthreads();
 
     if (a.split > 1) {
@@ -676,9 +710,10 @@ vsample_kernel(const __grid_constant__ VsArgs a)
                                                 a.part + 3 * (size_t)blockIdx.x);
     } else {
         CubeSums acc;
-        sample_cubes<FAM, MIXED, ADJ, NB4, D, FIX>(a, cells, hist, a.cube_begin, a.cube_end - a.cube_begin, a.perm_k,
+        sample_cubes<FAM, MIXED, ADJ, NB4, D, FIX>(a, cells, hist, a.cube_begin, a.cube_end - a.cube_begin, a.perm_k, a.perm_inv,
                                            blockIdx.x, gridDim.x, it, a.lanes, a.p, acc);
-        block_write_sums(acc, red, a.part + 3 * (size_t)blockIdx.x);
+        grid_dependents_launch();  // the refinement's blocks may take their places
+        block_write_sums<MIXED>(acc, a.want_abs != 0, red, a.part + 3 * (size_t)blockIdx.x);
     }
     if constexpr (ADJ) {
         __syncthreads();
@@ -729,8 +764,7 @@ cudaError_t launch_vsample_family(bool mixed, bool adjust, const VsArgs& a, int 
     auto k = vsample_kernel_ptr<FAM>(mixed, adjust, a.fam.fix != 0, (int)a.d);
     cudaError_t e = raise_smem_limit((const void*)k, smem);
     if (e != cudaSuccess) return e;
-    k<<<grid, vsample_threads(FAM, mixed, (int)a.d), smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(k, grid, vsample_threads(FAM, mixed, (int)a.d), smem, s, a);
 }
 
 template <int FAM>
