@@ -242,7 +242,7 @@ void BatchEngine::release()
 size_t BatchEngine::smem_bytes(int cls) const
 {
     const int dcls = cls % kDMax + 1;  // the class's dimension
-    return (size_t)dcls * opts_.nbins * (cell_bytes(mixed_) + hist_bytes(mixed_));
+    return (size_t)dcls * opts_.nbins * cell_bytes(mixed_) + hist_smem_bytes(mixed_, (uint32_t)(dcls * opts_.nbins));
 }
 
 int BatchEngine::class_blocks(int cls) const { return std::max(1, std::min(tuned_bps_, occ_[cls])) * num_sms_; }

@@ -34,6 +34,8 @@ vsample_batch_kernel(const __grid_constant__ BatchArgs a)
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double red[3][kVsThreads / 32];
     __shared__ __align__(16) BatchDesc sd;
+    __shared__ uint4 philox_tab[kPhiloxTab * NB4];
+    __shared__ uint32_t cube_step[2 * kDMax];
 
     const uint32_t s_begin = a.blk_seg[blockIdx.x], s_end = a.blk_seg[blockIdx.x + 1];
     for (uint32_t si = s_begin; si < s_end; ++si) {
@@ -55,20 +57,27 @@ vsample_batch_kernel(const __grid_constant__ BatchArgs a)
         if (threadIdx.x == 0) a.segs[si].adjust = adjust ? 1u : 0u;
         constexpr uint32_t d = D;
         const uint32_t nb = sd.nb;
-        Cell* cells = reinterpret_cast<Cell*>(smem);
-        HT* hist = reinterpret_cast<HT*>(smem + cell_bytes(MIXED) * d * nb);
+        HT* hist = reinterpret_cast<HT*>(smem + (MIXED ? 0u : cell_bytes(false) * d * nb));
+        Cell* cells = reinterpret_cast<Cell*>(smem + (MIXED ? hist_smem_bytes(true, d * nb) : 0u));
         if (adjust) clear_hist(hist, d * nb);
         stage_cells<MIXED>(cells, sd.cells, d, nb);
-        __syncthreads();
-
         const BatchView v{d,        nb,           sd.g,     sd.gmagic,         sd.key0,          sd.key1, d,
                           sd.jac0,  sd.phi_scale_f, sd.inv_p, sd.inv_var_den, sd.inv_p_f, sd.inv_var_den_f, 0u,
-                          sd.fam};
+                          cube_step, sd.fam};
         const uint32_t it = B.it;
+        fill_philox_table<NB4>(philox_tab, v, it);
+        const SampleRng<NB4> rng{it, philox_tab};
+        if (threadIdx.x == blockDim.x - 1) {
+            const uint64_t n = seg.c1 - seg.c0;
+            const uint64_t step = mod_by(mod_by(blockDim.x / sd.lanes, n, seg.perm_inv) * seg.perm_k, n, seg.perm_inv);
+            cube_step_digits32((uint32_t)step, (uint32_t)n, (uint32_t)sd.m, D, v, cube_step);
+        }
+        __syncthreads();
+
         CubeSums acc;
         auto sample = [&](auto adj_c, auto fix_c) {
             sample_cubes<FAM, MIXED, decltype(adj_c)::value, NB4, D, decltype(fix_c)::value>(
-                v, cells, hist, seg.c0, seg.c1 - seg.c0, seg.perm_k, seg.perm_inv, 0, 1, it, sd.lanes, sd.p, acc);
+                v, cells, hist, seg.c0, seg.c1 - seg.c0, seg.perm_k, seg.perm_inv, 0, 1, rng, sd.lanes, sd.p, acc);
         };
         bool done = false;
         if constexpr (!MIXED && FixFamily<FAM>::kHas) {

@@ -70,9 +70,7 @@ cudaError_t vsample_occupancy(int family, bool mixed, bool adjust, bool fix, int
 
 size_t vsample_smem_bytes(bool mixed, bool adjust, int d, int nb, int hist_d)
 {
-    const size_t cell = mixed ? 8 : 16;  // float2 or double2 cells
-    const size_t h = adjust ? (mixed ? 4 : 8) : 0;
-    return (size_t)d * nb * cell + (size_t)hist_d * nb * h;
+    return (size_t)d * nb * cell_bytes(mixed) + (adjust ? hist_smem_bytes(mixed, (uint32_t)(hist_d * nb)) : 0);
 }
 
 // ---------------------------------------------------------------------------
@@ -539,7 +537,9 @@ mcubes_status mcubes_setup(mcubes_ctx* c, int id, const double* params, int npar
     c->smem_noadj = vsample_smem_bytes(c->mixed, false, d, nb, c->hist_d);
     int smem_limit = 0;
     MC_CHECK(c, cudaDeviceGetAttribute(&smem_limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
-    if (c->smem_adj + 1024 > (size_t)smem_limit) return MCUBES_EINVAL;  // grid + histogram must fit on chip
+    // grid + histogram must fit on chip (1 KB covers the kernel's own arrays and the histogram's rounding)
+    const size_t on_chip = (size_t)d * nb * cell_bytes(c->mixed) + (size_t)c->hist_d * nb * hist_bytes(c->mixed);
+    if (on_chip + 1024 > (size_t)smem_limit) return MCUBES_EINVAL;
     int occ_adj = 0, occ_noadj = 0;
     MC_CHECK(c, vsample_occupancy(id, c->mixed, true, fp.fix != 0, d, c->smem_adj, &occ_adj));
     MC_CHECK(c, vsample_occupancy(id, c->mixed, false, fp.fix != 0, d, c->smem_noadj, &occ_noadj));

@@ -29,35 +29,20 @@ struct DD {
 // ---------------------------------------------------------------------------
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, "Parallel random numbers: as easy
 // as 1, 2, 3", SC'11).  The round keys (key + r * Weyl increments) are
-// precomputed on the host and read from the kernel's constant bank.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint4 philox4x32_10(uint4 x, const uint32_t (&rk)[10][2])
-{
-#pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        const uint32_t a0 = x.x * 0xD2511F53u, h0 = __umulhi(x.x, 0xD2511F53u);
-        const uint32_t a1 = x.z * 0xCD9E8D57u, h1 = __umulhi(x.z, 0xCD9E8D57u);
-        x = make_uint4(h1 ^ x.y ^ rk[r][0], a1, h0 ^ x.w ^ rk[r][1], a0);
-    }
-    return x;
-}
+// precomputed on the host and read from the kernel's constant bank (single
+// integrals) or formed from the integral's key (batches).
+//
+// The counter of a sample's block is (sample s, cube c, iteration it, block b),
+// and the first three rounds mix those words only in part: with one word of
+// the state multiplied per half and round, rounds 1-3 are products of it, of
+// s (and b) and of c alone, and of one word of (c, s).  So they are taken
+// apart: the products of (it, s, b) once per launch and segment for the first
+// samples of a cube (philox_shared, kept in shared memory), that of c once
+// per cube (PhiloxCube), that of (c, s) once per sample, and a block starts
+// at round 4: 30 instructions instead of 40.
+constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
 
-// The same generator with the round keys formed on the fly from the key
-// (for kernels whose key is per-integral data rather than a launch constant).
-__device__ __forceinline__ uint4 philox4x32_10_key(uint4 x, uint32_t k0, uint32_t k1)
-{
-#pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        const uint32_t a0 = x.x * 0xD2511F53u, h0 = __umulhi(x.x, 0xD2511F53u);
-        const uint32_t a1 = x.z * 0xCD9E8D57u, h1 = __umulhi(x.z, 0xCD9E8D57u);
-        x = make_uint4(h1 ^ x.y ^ k0, a1, h0 ^ x.w ^ k1, a0);
-        k0 += 0x9E3779B9u;
-        k1 += 0xBB67AE85u;
-    }
-    return x;
-}
-
-__device__ __forceinline__ uint4 sample_words(const VsArgs& a, uint4 ctr) { return philox4x32_10(ctr, a.rk); }
+__device__ __forceinline__ uint32_t round_key(const VsArgs& a, int r, int i) { return a.rk[r][i]; }
 
 // Register view of one batch integral for the per-sample code (the family
 // constants stay in shared memory).
@@ -69,12 +54,92 @@ struct BatchView {
     double inv_p, inv_var_den;     // 1/p, 1/(p (p-1))
     float inv_p_f, inv_var_den_f;
     uint32_t want_abs;             // 0: a batch iteration does not use the sums of |cube mean|
+    const uint32_t* cube_step;     // shared memory: [2][kDMax] digits of the cube step (cube_step_digit)
     const FamParams& fam;
 };
 
-__device__ __forceinline__ uint4 sample_words(const BatchView& v, uint4 ctr)
+// The keys grow by Weyl increments from the integral's own key.
+__device__ __forceinline__ uint32_t round_key(const BatchView& v, int r, int i)
 {
-    return philox4x32_10_key(ctr, v.key0, v.key1);
+    return i == 0 ? v.key0 + (uint32_t)r * 0x9E3779B9u : v.key1 + (uint32_t)r * 0xBB67AE85u;
+}
+
+// What rounds 1-3 make of (it, s, b) alone, the keys folded in.
+template <class A>
+__device__ __forceinline__ uint4 philox_shared(const A& a, uint32_t it, uint32_t s, uint32_t b)
+{
+    const uint32_t y1 = it * kPhiloxM1;
+    const uint32_t z1 = __umulhi(s, kPhiloxM0) ^ b ^ round_key(a, 0, 1);
+    const uint32_t x2 = __umulhi(z1, kPhiloxM1) ^ y1 ^ round_key(a, 1, 0);
+    return make_uint4((z1 * kPhiloxM1) ^ round_key(a, 2, 0), __umulhi(x2, kPhiloxM0) ^ round_key(a, 2, 1),
+                      (x2 * kPhiloxM0) ^ round_key(a, 3, 1), (s * kPhiloxM0) ^ round_key(a, 1, 1));
+}
+
+// What rounds 1 and 2 make of (it, c).
+struct PhiloxCube {
+    uint32_t h, l;
+};
+template <class A>
+__device__ __forceinline__ PhiloxCube philox_cube(const A& a, uint32_t it, uint32_t c)
+{
+    const uint32_t x1 = __umulhi(it, kPhiloxM1) ^ c ^ round_key(a, 0, 0);
+    return PhiloxCube{__umulhi(x1, kPhiloxM0), x1 * kPhiloxM0};
+}
+
+// The sample's word of rounds 2 and 3, from the cube's and the shared word w.
+__device__ __forceinline__ PhiloxCube philox_sample(const PhiloxCube& pc, uint32_t w)
+{
+    const uint32_t z2 = pc.h ^ w;
+    return PhiloxCube{__umulhi(z2, kPhiloxM1), z2 * kPhiloxM1};
+}
+
+// Rounds 4-10 of one block: u of the block (philox_shared), pc of the cube,
+// ps of the sample.
+template <class A>
+__device__ __forceinline__ uint4 philox_block(const A& a, const uint4& u, const PhiloxCube& pc, const PhiloxCube& ps)
+{
+    uint4 x = make_uint4(ps.h ^ u.x, 0u, u.y ^ pc.l, 0u);
+    {
+        const uint32_t a0 = x.x * kPhiloxM0, h0 = __umulhi(x.x, kPhiloxM0);
+        const uint32_t a1 = x.z * kPhiloxM1, h1 = __umulhi(x.z, kPhiloxM1);
+        x = make_uint4(h1 ^ ps.l ^ round_key(a, 3, 0), a1, h0 ^ u.z, a0);
+    }
+#pragma unroll
+    for (int r = 4; r < 10; ++r) {
+        const uint32_t a0 = x.x * kPhiloxM0, h0 = __umulhi(x.x, kPhiloxM0);
+        const uint32_t a1 = x.z * kPhiloxM1, h1 = __umulhi(x.z, kPhiloxM1);
+        x = make_uint4(h1 ^ x.y ^ round_key(a, r, 0), a1, h0 ^ x.w ^ round_key(a, r, 1), a0);
+    }
+    return x;
+}
+
+// A launch's (segment's) random words: the shared parts of its first kPhiloxTab
+// samples per cube in shared memory ([sample][block]), of later ones formed
+// where they are used.
+constexpr uint32_t kPhiloxTab = 4;
+template <int NB4> struct SampleRng {
+    uint32_t it;
+    const uint4* tab;
+    template <class A> __device__ uint4 shared_words(const A& a, uint32_t s, uint32_t b) const
+    {
+        return s < kPhiloxTab ? tab[s * NB4 + b] : philox_shared(a, it, s, b);
+    }
+};
+template <int NB4, class A>
+__device__ __forceinline__ void fill_philox_table(uint4* tab, const A& a, uint32_t it)
+{
+    if (threadIdx.x < kPhiloxTab * NB4) tab[threadIdx.x] = philox_shared(a, it, threadIdx.x / NB4, threadIdx.x % NB4);
+}
+
+// Digit of the cube step on axis j times nb; wrap: of the step that also takes
+// the range's length off (both modulo the number of cubes).
+__device__ __forceinline__ uint32_t cube_step_digit(const VsArgs& a, bool wrap, int j)
+{
+    return wrap ? a.cube_step[1][j] : a.cube_step[0][j];
+}
+__device__ __forceinline__ uint32_t cube_step_digit(const BatchView& v, bool wrap, int j)
+{
+    return v.cube_step[(wrap ? kDMax : 0) + j];
 }
 
 // ---------------------------------------------------------------------------
@@ -256,25 +321,29 @@ __device__ __forceinline__ DD edge_left(const double* row, const double* row_lo,
 //     nb y = (Q + a_lo 2^-33) / g,   k = floor(Q / g),
 //     phi = nb y - k = (Q mod g + a_lo 2^-33) / g.
 // Q < nb g <= 2^31, so floor(Q/g) is one high multiply by
-// gmagic = floor((2^32-1)/g) and at most one correction.
+// gmagic = floor((2^32-1)/g) and at most one correction.  With
+// (Q + 1) gmagic = (Q + 1) 2^32 / g - (Q + 1) e / g, 1 <= e <= g, the high
+// word of (Q + 1) gmagic is floor(Q/g) itself wherever nb g^2 <= 2^32: always
+// for d >= 3, where g^3 < 2^32 and nb <= 1024.  There Q + 1 is kept (the
+// cube's nb c carries the 1) and no correction is made (kExact).
 // ---------------------------------------------------------------------------
-struct BinPos {
+template <bool kExact> struct BinPos {
     uint32_t k;    // bin index
-    uint32_t r;    // Q mod g
+    uint32_t r;    // Q mod g (kExact: plus 1)
     uint32_t ahi;  // bit 32 of a_lo (i.e. A >> 32 & 1)
     uint32_t alo;  // low 32 bits of a_lo
 };
 
-__device__ __forceinline__ BinPos bin_pos(uint32_t w, uint32_t nb_c, uint32_t nb, uint32_t g,
-                                          uint32_t gmagic)
+template <bool kExact>
+__device__ __forceinline__ BinPos<kExact> bin_pos(uint32_t w, uint32_t nb_c, uint32_t nb, uint32_t g, uint32_t gmagic)
 {
     const uint64_t A = (uint64_t)(2u * nb) * (uint64_t)w + (uint64_t)nb;
     const uint32_t hi = (uint32_t)(A >> 32);
     const uint32_t Q = nb_c + (hi >> 1);
     uint32_t q = __umulhi(Q, gmagic);
     uint32_t r = Q - q * g;
-    if (r >= g) { ++q; r -= g; }
-    BinPos b;
+    if (!kExact && r >= g) { ++q; r -= g; }
+    BinPos<kExact> b;
     b.k = q;
     b.r = r;
     b.ahi = hi & 1u;
@@ -282,14 +351,21 @@ __device__ __forceinline__ BinPos bin_pos(uint32_t w, uint32_t nb_c, uint32_t nb
     return b;
 }
 
+// r 2^33 + a_lo, the numerator of g phi 2^33
+template <bool kExact> __device__ __forceinline__ uint64_t bin_numerator(const BinPos<kExact>& b)
+{
+    const uint32_t hi = kExact ? b.r + b.r + b.ahi - 2u : (b.r << 1) | b.ahi;
+    return ((uint64_t)hi << 32) | (uint64_t)b.alo;  // < 2^63
+}
+
 // g phi = r + a_lo 2^-33 as a double, built from the integer numerator
 // r 2^33 + a_lo with integer operations only (exact below 2^53, rounded to
 // nearest above): no FP64 conversion or multiply in the sampling loop.  The
 // numerator is never 0: its low 33 bits are those of A = nb (2w + 1), an odd
 // multiple of nb < 2^33.
-__device__ __forceinline__ double bin_gphi_f64(const BinPos& b)
+template <bool kExact> __device__ __forceinline__ double bin_gphi_f64(const BinPos<kExact>& b)
 {
-    const uint64_t num = ((uint64_t)b.r << 33) | ((uint64_t)b.ahi << 32) | (uint64_t)b.alo;  // < 2^63
+    const uint64_t num = bin_numerator(b);
     const int lz = __clzll((long long)num);
     uint64_t m;  // num with its leading one moved to bit 52 (bit 53 after a rounding carry)
     if (lz >= 11) {
@@ -305,9 +381,11 @@ __device__ __forceinline__ double bin_gphi_f64(const BinPos& b)
 }
 
 // the same in single precision: (r + a_lo 2^-33) * scale, scale = 1/g for phi
-__device__ __forceinline__ float bin_phi_f32(const BinPos& b, float scale)
+// (kExact: r + 1 <= 2^11, so taking 1 off in single precision is exact)
+template <bool kExact> __device__ __forceinline__ float bin_phi_f32(const BinPos<kExact>& b, float scale)
 {
-    const float base = __uint2float_rn(b.r) + (b.ahi ? 0.5f : 0.0f);
+    const float base = kExact ? __uint2float_rn(b.r) + (b.ahi ? -0.5f : -1.0f)
+                              : __uint2float_rn(b.r) + (b.ahi ? 0.5f : 0.0f);
     return __fmul_rn(__fmaf_rn(__uint2float_rn(b.alo), 1.16415321826934814453125e-10f /*2^-33*/, base), scale);
 }
 

@@ -29,7 +29,9 @@ constexpr int kVsThreadsMax = 1024; // largest block of a single-integral sampli
 constexpr int kCosmo6Threads = 1024;
 __host__ __device__ constexpr int vsample_threads(int family, bool mixed, int d)
 {
-    return (family == MCUBES_F_COSMO6 && !mixed && d == 6) ? kCosmo6Threads : kVsThreads;
+    if (mixed || family == MCUBES_F_TABLE) return kVsThreads;
+    if (family == MCUBES_F_COSMO6) return d == 6 ? kCosmo6Threads : kVsThreads;
+    return d <= 6 ? kVsThreads : d <= 6 ? 256 : d <= 9 ? 384 : 768;
 }
 constexpr int kRefineThreads = 512;
 
@@ -37,6 +39,11 @@ constexpr int kRefineThreads = 512;
 // edge, nb * width) in double or single precision, and a histogram entry.
 __host__ __device__ constexpr size_t cell_bytes(bool mixed) { return mixed ? 8 : 16; }
 __host__ __device__ constexpr size_t hist_bytes(bool mixed) { return mixed ? 4 : 8; }
+// A block's histogram of n bins, rounded up to the cells' 16-byte alignment.
+__host__ __device__ constexpr uint32_t hist_smem_bytes(bool mixed, uint32_t n)
+{
+    return (n * (uint32_t)hist_bytes(mixed) + 15u) & ~15u;
+}
 
 // Per-integral state kept on the device across iterations, so that the whole
 // iteration loop (sample -> refine -> weight -> converge) runs without the
@@ -117,6 +124,8 @@ struct VsArgs {
     uint64_t cube_begin, cube_end;
     uint64_t perm_k;          // cube order: logical i -> cube_begin + (i perm_k mod n), gcd(perm_k, n) = 1
     uint64_t perm_inv;        // floor((2^64 - 1) / n) (set_cube_order sets both)
+    uint32_t cube_step[2][kDMax];  // digits times nb of the step from a block's group of cubes to its next one,
+                                   // and of the step that wraps around the range (set by launch_vsample)
     uint32_t rk[10][2];       // Philox round keys (key + r * Weyl constants)
     double lo[kDMax];
     double scale[kDMax];      // hi - lo
@@ -275,6 +284,20 @@ template <class T> void set_cube_order(T& a, uint64_t n)  // of a range of n cub
 {
     a.perm_k = cube_permutation(n);
     a.perm_inv = n ? ~0ull / n : 0ull;
+}
+// Digits (times nb, axis 0 fastest) of the cube steps of a range of n of m = g^d
+// cubes walked in groups of `group` logical cubes: [0] the step (group perm_k
+// mod n), [1] the step less n, modulo m.
+inline void cube_step_digits(uint64_t step, uint64_t n, uint64_t m, uint32_t d, uint32_t g,
+                                                 uint32_t nb, uint32_t* plain, uint32_t* wrapped)
+{
+    uint64_t u = step, v = step + (m - n);  // step < n <= m: v < m
+    for (uint32_t j = 0; j < d; ++j) {
+        plain[j] = (uint32_t)(u % g) * nb;
+        wrapped[j] = (uint32_t)(v % g) * nb;
+        u /= g;
+        v /= g;
+    }
 }
 // Raises a kernel's dynamic shared-memory limit on the current device to at
 // least smem bytes (never lowers it, so that contexts of different sizes can

@@ -24,90 +24,84 @@
 
 namespace mc {
 
-// Adds v to the shared-memory histogram word at byte offset `off` of the
-// histogram whose shared-window address is `base` (a reduction: no value
-// comes back, so nothing waits on it).
+// The flat bin indices of a sample's axes are kept two per word, axis 2k in the
+// low half of word k: as they are in double precision, as byte offsets into the
+// histogram (4 times the index, below 2^16 as 12 x 1024 bins take 48 KB) in
+// single precision.  An odd last axis leaves the top half kNoBin.
+constexpr uint32_t kNoBin = 0xFFFFu;
+template <class HT> constexpr uint32_t bin_unit() { return sizeof(HT) == 4 ? 4u : 1u; }
+
+// Adds v to the bin at `idx` (bin_unit) of the shared-memory histogram at
+// shared-window address `base` (a reduction: no value comes back, so nothing
+// waits on it).
 __device__ __forceinline__ void hist_add(uint32_t base, uint32_t idx, float v)
 {
-    asm volatile("red.shared.add.f32 [%0], %1;" ::"r"(base + 4u * idx), "f"(v));
+    asm volatile("red.shared.add.f32 [%0], %1;" ::"r"(base + idx), "f"(v));
 }
 __device__ __forceinline__ void hist_add(uint32_t base, uint32_t idx, double v)
 {
     asm volatile("red.shared.add.f64 [%0], %1;" ::"r"(base + 8u * idx), "d"(v));
 }
 
-// Adds F2 to the sample's bin on each of the first hist_d axes; idx holds the
-// flat bin indices two per word (axis 2k in the low half of idx[k]).  In
-// double precision, where a shared-memory add is a compare-and-swap loop that
-// repeats while lanes of the warp collide on one bin, odd lanes take the two
-// axes of each word in the opposite order: at every step the warp adds to two
-// different axes' histograms and half as many lanes compete for the same
-// bins.  The single-precision add is a native reduction; there the swap
-// measured slower and is not made.
-template <int NB4, class HT>
-__device__ __forceinline__ void hist_add_sample(uint32_t hist_s, const uint32_t (&idx)[2 * NB4], uint32_t hist_d,
-                                                HT F2)
+// Adds F2 to the sample's bin on every axis.  A shared-memory float addition
+// is a compare-and-swap loop that repeats for the whole warp while lanes
+// collide on one bin, so from three axes on the lanes start at different words
+// and take the words in turn from there, NW = ceil(DC/2) words in all.  In
+// double precision lane pair t (lanes 2t, 2t+1) starts at word (t mod NW), the
+// odd lane of the pair with the two halves swapped, so each of the NW steps
+// adds to 2 NW different axes' histograms, about 32 / (2 NW) lanes each,
+// instead of two axes with 16 lanes each; in single precision lane l starts at
+// word (l mod NW), no halves swapped (measured faster: corner8 17.57 -> 17.42
+// ms, osc10 21.69 -> 21.00 ms per 1e9-call pass, against 17.65 and 21.33 with
+// the swap).  The words are rotated by selects, a power of two at a time
+// (static register indices).
+template <int DC, int NB4, class HT>
+__device__ __forceinline__ void hist_add_all(uint32_t hist_s, const uint32_t (&idx)[2 * NB4], HT F2)
 {
-    const uint32_t odd = sizeof(HT) == 8 ? (threadIdx.x & 1u) : 0u;
-#pragma unroll
-    for (int k = 0; k < 2 * NB4; ++k) {
-        if (2 * k < (int)hist_d) {
-            const uint32_t w = __funnelshift_l(idx[k], idx[k], odd << 4);  // halves swapped on odd lanes
-            if (((2u * k) ^ odd) < hist_d) hist_add(hist_s, w & 0xFFFFu, F2);
-            if (((2u * k + 1u) ^ odd) < hist_d) hist_add(hist_s, w >> 16, F2);
-        }
-    }
-}
-
-// The same for a sample of DC axes, every one with a histogram (hist_d =
-// DC): the lanes start at different index words and take the words in turn
-// from there, NW = ceil(DC/2) words in all.  In double precision lane pair t
-// (lanes 2t, 2t+1) starts at word (t mod NW), the odd lane of the pair with
-// the two halves swapped as above, so each of the NW steps adds to 2 NW
-// different axes' histograms, about 32 / (2 NW) lanes each, instead of two
-// axes with 16 lanes each; in single precision lane l starts at word
-// (l mod NW), no halves swapped (measured faster: corner8 17.57 -> 17.42 ms,
-// osc10 21.69 -> 21.00 ms per 1e9-call pass, against 17.65 and 21.33 with
-// the swap).  Fewer lanes of a warp collide on one bin, and each collision
-// repeats the shared-memory compare-and-swap for the whole warp.  The words
-// are picked with selects (static register indices).
-template <int NW, int NB4, class HT>
-__device__ __forceinline__ void hist_add_sample_rotated(uint32_t hist_s, const uint32_t (&idx)[2 * NB4],
-                                                        uint32_t hist_d, HT F2)
-{
-    static_assert(NW >= 2 && NW <= 2 * NB4, "rotation over the words in use");
+    constexpr int NW = (DC + 1) / 2;
     constexpr bool kSwap = sizeof(HT) == 8;
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t odd = kSwap ? (lane & 1u) : 0u;
-    const uint32_t rot = (kSwap ? (lane >> 1) : lane) % (uint32_t)NW;
+    uint32_t w[NW];
+#pragma unroll
+    for (int t = 0; t < NW; ++t) w[t] = idx[t];
+    if constexpr (NW >= 2) {
+        const uint32_t rot = (kSwap ? (lane >> 1) : lane) % (uint32_t)NW;
+#pragma unroll
+        for (int sh = 1; sh < NW; sh <<= 1) {
+            const bool on = (rot & (uint32_t)sh) != 0u;
+            uint32_t u[NW];
+#pragma unroll
+            for (int t = 0; t < NW; ++t) u[t] = on ? w[(t + sh) % NW] : w[t];
+#pragma unroll
+            for (int t = 0; t < NW; ++t) w[t] = u[t];
+        }
+    }
 #pragma unroll
     for (int t = 0; t < NW; ++t) {
-        uint32_t w = idx[t], k = (uint32_t)t;
-#pragma unroll
-        for (int q = 1; q < NW; ++q) {
-            if (rot == (uint32_t)q) {
-                w = idx[(t + q) % NW];
-                k = (uint32_t)((t + q) % NW);
-            }
-        }
-        w = __funnelshift_l(w, w, odd << 4);  // halves swapped on odd lanes
-        if (((2u * k) ^ odd) < hist_d) hist_add(hist_s, w & 0xFFFFu, F2);
-        if (((2u * k + 1u) ^ odd) < hist_d) hist_add(hist_s, w >> 16, F2);
+        const uint32_t v = kSwap ? __funnelshift_l(w[t], w[t], odd << 4) : w[t];  // halves swapped on odd lanes
+        const uint32_t lo = v & 0xFFFFu, hi = v >> 16;
+        if (!(DC & 1) || !kSwap || lo != kNoBin) hist_add(hist_s, lo, F2);
+        if (!(DC & 1) || hi != kNoBin) hist_add(hist_s, hi, F2);
     }
 }
 
-// The histogram adds of one sample: rotated where the axis count is a
-// compile-time DC >= 3 with a histogram on every axis.
+// The histogram adds of one sample: on all DC axes, or on axis 0 alone
+// (m-Cubes1D, Sec. 3).
 template <int DC, int NB4, class HT>
 __device__ __forceinline__ void hist_add_one(uint32_t hist_s, const uint32_t (&idx)[2 * NB4], uint32_t hist_d, HT F2)
 {
-    if constexpr (DC >= 3) {
-        if (hist_d == (uint32_t)DC) {
-            hist_add_sample_rotated<(DC + 1) / 2, NB4, HT>(hist_s, idx, hist_d, F2);
-            return;
-        }
-    }
-    hist_add_sample<NB4>(hist_s, idx, hist_d, F2);
+    if (hist_d == (uint32_t)DC) hist_add_all<DC, NB4, HT>(hist_s, idx, F2);
+    else hist_add(hist_s, idx[0] & 0xFFFFu, F2);
+}
+
+// Packs axis j's bin into the index words.
+template <int DC, class HT, int NW>
+__device__ __forceinline__ void pack_bin(uint32_t (&idx)[NW], int j, uint32_t flat)
+{
+    const uint32_t v = flat * bin_unit<HT>();
+    if (j & 1) idx[j >> 1] |= v << 16;
+    else idx[j >> 1] = j == DC - 1 ? v | (kNoBin << 16) : v;
 }
 
 template <bool MIXED> struct Prec;
@@ -198,8 +192,8 @@ constexpr bool rolled_axes()
 // 9.55 and 9.69 ms against 8.80 ms per 1e8-call cosmo6 pass.)
 template <int FAM, bool MIXED, int NB4, int D, class A>
 __device__ __forceinline__ typename Prec<MIXED>::R
-sample_point_rolled(const A& a, const typename Prec<MIXED>::Cell* cells, uint32_t c, uint32_t s, uint32_t it,
-                    uint32_t (&idx)[2 * NB4])
+sample_point_rolled(const A& a, const typename Prec<MIXED>::Cell* cells, uint32_t c, uint32_t s,
+                    const SampleRng<NB4>& rng, const PhiloxCube& pc, uint32_t (&idx)[2 * NB4])
 {
     using R = typename Prec<MIXED>::R;
     using Fam = Family<FAM, R>;
@@ -210,13 +204,15 @@ sample_point_rolled(const A& a, const typename Prec<MIXED>::Cell* cells, uint32_
     R jac = R(1);          // mixed: single-precision product of the widths
     IntProd jp{0, 0};      // FP64: the product in integer arithmetic, from jac0
     if constexpr (!MIXED) jp = int_prod_of(a.jac0);
+    static_assert(D >= 3, "exact bin positions");
     uint32_t rest = c;
     uint4 r = make_uint4(0u, 0u, 0u, 0u);
+    const PhiloxCube ps = philox_sample(pc, rng.shared_words(a, s, 0).w);
 #pragma unroll
     for (int k = 0; k < 2 * NB4; ++k) idx[k] = 0u;
 #pragma unroll 1
     for (int j = 0; j < D; ++j) {
-        if ((j & 3) == 0) r = sample_words(a, make_uint4(s, c, it, (uint32_t)(j >> 2)));
+        if ((j & 3) == 0) r = philox_block(a, rng.shared_words(a, s, (uint32_t)(j >> 2)), pc, ps);
         const uint32_t w = r.x;
         r = make_uint4(r.y, r.z, r.w, r.x);
         uint32_t q = __umulhi(rest, a.gmagic);
@@ -224,7 +220,7 @@ sample_point_rolled(const A& a, const typename Prec<MIXED>::Cell* cells, uint32_
         if (dig >= a.g) { ++q; dig -= a.g; }
         if (dig >= a.g) { ++q; dig -= a.g; }
         rest = q;
-        const BinPos bp = bin_pos(w, dig * nb, nb, a.g, a.gmagic);
+        const BinPos<true> bp = bin_pos<true>(w, dig * nb + 1u, nb, a.g, a.gmagic);
         const uint32_t flat = (uint32_t)j * nb + bp.k;
         const auto cell = cells[flat];
         R x;
@@ -243,10 +239,28 @@ sample_point_rolled(const A& a, const typename Prec<MIXED>::Cell* cells, uint32_
     if constexpr (D & 1) {  // one field short of the top: move every field down once more
 #pragma unroll
         for (int k = 0; k < NW - 1; ++k) idx[k] = __funnelshift_r(idx[k], idx[k + 1], 16);
-        idx[NW - 1] >>= 16;
+        idx[NW - 1] = (idx[NW - 1] >> 16) | (kNoBin << 16);
     }
     if constexpr (!MIXED) return Fam::end_scaled(fs, a.fam, jp.m, jp.e);  // f J, rounded once
     else return Fam::end(fs, D, a.fam) * jac;
+}
+
+// The random words of a sample, four per Philox block.
+template <int NB4, class A>
+__device__ __forceinline__ void sample_words(const A& a, uint32_t s, const SampleRng<NB4>& rng, const PhiloxCube& pc,
+                                             uint32_t (&w)[4 * NB4])
+{
+    PhiloxCube ps;
+#pragma unroll
+    for (int b = 0; b < NB4; ++b) {
+        const uint4 u = rng.shared_words(a, s, (uint32_t)b);
+        if (b == 0) ps = philox_sample(pc, u.w);
+        const uint4 r = philox_block(a, u, pc, ps);
+        w[4 * b + 0] = r.x;
+        w[4 * b + 1] = r.y;
+        w[4 * b + 2] = r.z;
+        w[4 * b + 3] = r.w;
+    }
 }
 
 // The same sample in the fixed-point form (FixFamily): the cell holds t at
@@ -254,38 +268,30 @@ sample_point_rolled(const A& a, const typename Prec<MIXED>::Cell* cells, uint32_
 // 2^(e - 63); g phi = num 2^-33, num < g 2^33 shifted to the top of 64 bits by
 // fsg, so t = left + (M num 2^fsg) >> (64 + ftsh - e).
 template <int FAM, int NB4, int DC, class A>
-__device__ __forceinline__ double sample_point_fix(const A& a, const double2* cells, uint32_t c, uint32_t s,
-                                                   uint32_t it, const uint32_t (&nbc)[4 * NB4],
-                                                   uint32_t (&idx)[2 * NB4])
+__device__ __forceinline__ double sample_point_fix(const A& a, const double2* cells, uint32_t s,
+                                                   const SampleRng<NB4>& rng, const PhiloxCube& pc,
+                                                   const uint32_t (&nbc)[4 * NB4], uint32_t (&idx)[2 * NB4])
 {
     using Fam = FixFamily<FAM>;
     const uint32_t nb = a.nb;
     uint32_t w[4 * NB4];
-#pragma unroll
-    for (int b = 0; b < NB4; ++b) {
-        const uint4 r = sample_words(a, make_uint4(s, c, it, (uint32_t)b));
-        w[4 * b + 0] = r.x;
-        w[4 * b + 1] = r.y;
-        w[4 * b + 2] = r.z;
-        w[4 * b + 3] = r.w;
-    }
+    sample_words<NB4>(a, s, rng, pc, w);
     typename Fam::S fs;
     Fam::begin(fs, a.fam);
     IntProd jp = int_prod_of(a.jac0);
 #pragma unroll
     for (int j = 0; j < DC; ++j) {
-        const BinPos bp = bin_pos(w[j], nbc[j], nb, a.g, a.gmagic);
+        const auto bp = bin_pos<(DC >= 3)>(w[j], nbc[j], nb, a.g, a.gmagic);
         const uint32_t flat = (uint32_t)j * nb + bp.k;
         const double2 cell = cells[flat];
         const IntProd wd = int_prod_of(cell.y);
-        const uint64_t num = (((uint64_t)((bp.r << 1) | bp.ahi) << 32) | (uint64_t)bp.alo) << a.fam.fsg;
+        const uint64_t num = bin_numerator(bp) << a.fam.fsg;
         const uint64_t H = __umul64hi(wd.m, num);
         const uint32_t sh = (uint32_t)(a.fam.ftsh - wd.e);  // >= 0; beyond 63 for the narrowest bins
         const int64_t t = __double_as_longlong(cell.x) + (int64_t)(sh < 64u ? H >> sh : 0ull);
         jp = int_prod_mul2(jp, wd);
         Fam::add(fs, j, t, a.fam);
-        if (j & 1) idx[j >> 1] |= flat << 16;
-        else idx[j >> 1] = flat;
+        pack_bin<DC, double>(idx, j, flat);
     }
     return Fam::template end<DC>(fs, a.fam, jp);
 }
@@ -293,40 +299,32 @@ __device__ __forceinline__ double sample_point_fix(const A& a, const double2* ce
 // One sample: random words -> exact bin position -> map -> integrand.
 // Returns F = f(x) * J and leaves the flat histogram index of every axis in
 // idx (16 bits each, two per word).  A provides d, nb, g, gmagic, jac0 ((g nb)^d), phi_scale_f
-// (1/(g nb)), hist_d and fam, and sample_words(a, counter) its Philox block.
+// (1/(g nb)), hist_d and fam, and round_key(a, r, i) its Philox keys.
 template <int FAM, bool MIXED, int NB4, int DC, bool FIX, class A>
 __device__ __forceinline__ typename Prec<MIXED>::R
-sample_point(const A& a, const typename Prec<MIXED>::Cell* cells, uint32_t c, uint32_t s, uint32_t it,
-             const uint32_t (&nbc)[4 * NB4], uint32_t (&idx)[2 * NB4])
+sample_point(const A& a, const typename Prec<MIXED>::Cell* cells, uint32_t c, uint32_t s, const SampleRng<NB4>& rng,
+             const PhiloxCube& pc, const uint32_t (&nbc)[4 * NB4], uint32_t (&idx)[2 * NB4])
 {
     using R = typename Prec<MIXED>::R;
     using Fam = Family<FAM, R>;
-    if constexpr (FIX) return sample_point_fix<FAM, NB4, DC>(a, cells, c, s, it, nbc, idx);
-    if constexpr (DC > 0 && rolled_axes<FAM, MIXED>()) {
-        return sample_point_rolled<FAM, MIXED, NB4, DC>(a, cells, c, s, it, idx);
-    }
-    constexpr int DN = 4 * NB4;  // axes handled by this instantiation (d <= DN)
-    const uint32_t d = DC ? (uint32_t)DC : a.d, nb = a.nb;  // DC: the dimension when fixed at compile time
-    uint32_t w[DN];
-#pragma unroll
-    for (int b = 0; b < NB4; ++b) {
-        if (4 * b < (int)d) {
-            const uint4 r = sample_words(a, make_uint4(s, c, it, (uint32_t)b));
-            w[4 * b + 0] = r.x;
-            w[4 * b + 1] = r.y;
-            w[4 * b + 2] = r.z;
-            w[4 * b + 3] = r.w;
-        }
-    }
+    if constexpr (FIX) {
+        return sample_point_fix<FAM, NB4, DC>(a, cells, s, rng, pc, nbc, idx);
+    } else if constexpr (rolled_axes<FAM, MIXED>()) {
+        return sample_point_rolled<FAM, MIXED, NB4, DC>(a, cells, c, s, rng, pc, idx);
+    } else {
+    constexpr uint32_t d = DC;
+    const uint32_t nb = a.nb;
+    uint32_t w[4 * NB4];
+    sample_words<NB4>(a, s, rng, pc, w);
     typename Fam::S fs;
     Fam::begin(fs);
     R jac = R(1);                          // mixed: single-precision product of the widths
     IntProd jp{0, 0};                      // FP64: the product in integer arithmetic, from jac0
     if constexpr (!MIXED) jp = int_prod_of(a.jac0);
 #pragma unroll
-    for (int j = 0; j < DN; ++j) {
-        if (j < (int)d) {
-            const BinPos bp = bin_pos(w[j], nbc[j], nb, a.g, a.gmagic);
+    for (int j = 0; j < DC; ++j) {
+        {
+            const auto bp = bin_pos<(DC >= 3)>(w[j], nbc[j], nb, a.g, a.gmagic);
             const uint32_t flat = (uint32_t)j * nb + bp.k;
             const auto cell = cells[flat];
             R x;
@@ -339,13 +337,12 @@ sample_point(const A& a, const typename Prec<MIXED>::Cell* cells, uint32_t c, ui
             if constexpr (MIXED) jac *= cell.y;
             else int_prod_mul(jp, cell.y);
             Fam::add(fs, j, x, a.fam);
-            // flat histogram indices (< 2^16) packed two per register
-            if (j & 1) idx[j >> 1] |= flat << 16;
-            else idx[j >> 1] = flat;
+            pack_bin<DC, typename Prec<MIXED>::H>(idx, j, flat);
         }
     }
     if constexpr (!MIXED) jac = int_prod_value(jp);
     return Fam::end(fs, d, a.fam) * jac;
+    }
 }
 
 // Per-thread sums over the cubes a thread finishes: double, or a compensated
@@ -369,26 +366,81 @@ __device__ __forceinline__ uint64_t mod_by(uint64_t x, uint64_t n, uint64_t inv)
     return r;
 }
 
+// nb times the digit of cube c on every axis (axis 0 fastest), plus 1 where bin
+// positions are exact (bin_pos).
+template <int NB4, int DC, class A>
+__device__ __forceinline__ void cube_digits(const A& a, uint32_t c, uint32_t (&nbc)[4 * NB4])
+{
+    uint32_t rest = c;
+#pragma unroll
+    for (int j = 0; j < DC; ++j) {
+        uint32_t q = __umulhi(rest, a.gmagic);
+        uint32_t r = rest - q * a.g;
+        if (r >= a.g) { ++q; r -= a.g; }
+        if (r >= a.g) { ++q; r -= a.g; }
+        nbc[j] = r * a.nb + (DC >= 3 ? 1u : 0u);
+        rest = q;
+    }
+}
+
+// Adds the cube step's digits to a cube's, with carries (the last one drops:
+// cube indices are taken modulo g^d): four instructions per axis against ten
+// for splitting the new index by divisions.
+template <int NB4, int DC, class A>
+__device__ __forceinline__ void advance_digits(const A& a, bool wrap, uint32_t (&nbc)[4 * NB4])
+{
+    const uint32_t nb = a.nb, ng = nb * a.g, top = ng + (DC >= 3 ? 1u : 0u);
+    uint32_t carry = 0;
+#pragma unroll
+    for (int j = 0; j < DC; ++j) {
+        const uint32_t t = nbc[j] + cube_step_digit(a, wrap, j) + carry;  // < 2 ng <= 2^32
+        const bool over = t >= top;
+        nbc[j] = over ? t - ng : t;
+        carry = over ? nb : 0u;
+    }
+}
+
+// The digits of a segment's cube step into shared memory (cube_step_digits on
+// the device, 32-bit: one thread, D high multiplies each).
+template <class A>
+__device__ __forceinline__ void cube_step_digits32(uint32_t step, uint32_t n, uint32_t m, uint32_t d, const A& a,
+                                                   uint32_t* out)
+{
+    uint32_t u[2] = {step, step + (m - n)};
+#pragma unroll 1
+    for (uint32_t j = 0; j < d; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint32_t q = __umulhi(u[h], a.gmagic);
+            uint32_t rem = u[h] - q * a.g;
+            if (rem >= a.g) { ++q; rem -= a.g; }
+            if (rem >= a.g) { ++q; rem -= a.g; }
+            out[h * kDMax + j] = rem * a.nb;
+            u[h] = q;
+        }
+}
+
 // Samples cubes [cube_lo, cube_lo + ncubes) of one integral.  The block takes
 // groups of (blockDim / lanes) logical cube indices: group0, group0 + gstride,
 // ...; logical index i is cube cube_lo + (i * perm_k mod ncubes), a bijection
 // of the range (gcd(perm_k, ncubes) = 1) that gives the lanes of a warp
 // cubes with unrelated digits on every axis, so that their samples spread
 // over all bins instead of crowding the same few (fewer shared-memory atomic
-// conflicts and bank conflicts).  Besides what sample_point reads, A provides
-// inv_p = 1/p and inv_var_den = 1/(p (p-1)) (inv_p_f, inv_var_den_f in single
-// precision) and want_abs (whether the sums of |cube mean| are needed: they
-// are reported by the sampling-pass calls, not used by an iteration).
+// conflicts and bank conflicts).  From group to group a thread's cube moves by
+// one fixed step (or that step less ncubes), whose digits cube_step_digit(a)
+// gives.  Besides what sample_point reads, A provides inv_p = 1/p and
+// inv_var_den = 1/(p (p-1)) (inv_p_f, inv_var_den_f in single precision) and
+// want_abs (whether the sums of |cube mean| are needed: they are reported by
+// the sampling-pass calls, not used by an iteration).
 template <int FAM, bool MIXED, bool ADJ, int NB4, int DC, bool FIX, class A>
 __device__ __forceinline__ void sample_cubes(const A& a, const typename Prec<MIXED>::Cell* cells,
                                              typename Prec<MIXED>::H* hist, uint64_t cube_lo, uint64_t ncubes,
                                              uint64_t perm_k, uint64_t perm_inv, uint64_t group0, uint64_t gstride,
-                                             uint32_t it, uint32_t lanes, uint32_t p, CubeSums& acc)
+                                             const SampleRng<NB4>& rng, uint32_t lanes, uint32_t p, CubeSums& acc)
 {
     using R = typename Prec<MIXED>::R;
     using HT = typename Prec<MIXED>::H;
-    constexpr int DN = 4 * NB4;
-    const uint32_t d = DC ? (uint32_t)DC : a.d, nb = a.nb;
+    constexpr bool kRolled = !FIX && rolled_axes<FAM, MIXED>();  // peels its digits itself
     const uint32_t hist_d = a.hist_d;  // axes with a histogram: d, or 1 (m-Cubes1D, Sec. 3)
     const uint32_t hist_s = (uint32_t)__cvta_generic_to_shared(hist);
     const uint32_t L = lanes;
@@ -406,40 +458,64 @@ __device__ __forceinline__ void sample_cubes(const A& a, const typename Prec<MIX
         inv_var_den = a.inv_var_den;
     }
     const uint64_t first = group0 * cubes_per_group + threadIdx.x / L;
+    const uint64_t stride = gstride * cubes_per_group;
     // physical offset of `first`, and its step from group to group (below 2^32, as the cube counter)
     uint32_t off = (uint32_t)mod_by(mod_by(first, ncubes, perm_inv) * perm_k, ncubes, perm_inv);
-    const uint32_t step =
-        (uint32_t)mod_by(mod_by(gstride * cubes_per_group, ncubes, perm_inv) * perm_k, ncubes, perm_inv);
-    for (uint64_t base = group0 * cubes_per_group; base < ncubes; base += gstride * cubes_per_group) {
-        const uint64_t ci = base + threadIdx.x / L;
-        const bool valid = ci < ncubes;
-        const uint32_t c = (uint32_t)cube_lo + (valid ? off : 0u);
+    const uint32_t step = (uint32_t)mod_by(mod_by(stride, ncubes, perm_inv) * perm_k, ncubes, perm_inv);
+    uint32_t nbc[4 * NB4];
+    if constexpr (!kRolled) cube_digits<NB4, DC>(a, (uint32_t)cube_lo + off, nbc);
+    auto advance = [&] {  // to this thread's cube of the next group
         off += step;
-        if (off < step || off >= (uint32_t)ncubes) off -= (uint32_t)ncubes;
-        // sub-cube digits (axis 0 fastest), kept as nb * digit
-        uint32_t nbc[DN];
-        {
-            uint32_t rest = c;
-#pragma unroll
-            for (int j = 0; j < DN; ++j) {
-                if (j < (int)d) {
-                    uint32_t q = __umulhi(rest, a.gmagic);
-                    uint32_t r = rest - q * a.g;
-                    if (r >= a.g) { ++q; r -= a.g; }
-                    if (r >= a.g) { ++q; r -= a.g; }
-                    nbc[j] = r * nb;
-                    rest = q;
-                }
+        const bool wrap = off < step || off >= (uint32_t)ncubes;
+        if (wrap) off -= (uint32_t)ncubes;
+        if constexpr (!kRolled) advance_digits<NB4, DC>(a, wrap, nbc);
+    };
+    if (L == 1u && p == 2u) {
+        // two samples per cube, one thread each (every 1e8-call geometry)
+        for (uint64_t ci = first; ci < ncubes; ci += stride) {
+            const uint32_t c = (uint32_t)cube_lo + off;
+            const PhiloxCube pc = philox_cube(a, rng.it, c);
+            R K = R(0), F = R(0);
+#pragma unroll 1
+            for (uint32_t s = 0; s < 2u; ++s) {
+                uint32_t idx[2 * NB4];
+                K = F;
+                F = sample_point<FAM, MIXED, NB4, DC, FIX>(a, cells, c, s, rng, pc, nbc, idx);
+                if constexpr (ADJ) hist_add_one<DC, NB4>(hist_s, idx, hist_d, (HT)(F * F));
+            }
+            advance();
+            // UpdateVariance (Alg. 3): cube mean and the variance of that mean;
+            // S1 = z, S2 = z^2 and the variance (z^2 - z^2/2)/2 is exactly z^2/4:
+            // the z^2 are summed and the sum scaled once after the loop (exact)
+            const RS S1 = (RS)F - (RS)K;
+            const RS mean = (RS)K + S1 * RS(0.5);
+            if constexpr (sizeof(RS) == 4) {
+                acc.fI.add(mean);
+                acc.fV.add(S1 * S1);
+                if (a.want_abs) acc.fA.add(fabsf(mean));
+            } else {
+                acc.I += mean;
+                acc.V = fma(S1, S1, acc.V);  // one FMA for the z^2
+                if (a.want_abs) acc.A += fabs(mean);
             }
         }
+        acc.V *= 0.25;
+        acc.fV.hi *= 0.25f;
+        acc.fV.lo *= 0.25f;
+        return;
+    }
+    for (uint64_t base = group0 * cubes_per_group; base < ncubes; base += stride) {
+        const bool valid = base + threadIdx.x / L < ncubes;
+        const uint32_t c = (uint32_t)cube_lo + off;
         // this lane's samples of the cube, shifted by its first value
         R K = R(0);
         RS S1 = RS(0), S2 = RS(0);
         uint32_t n = 0;
         if (valid) {
+            const PhiloxCube pc = philox_cube(a, rng.it, c);
             for (uint32_t s = seg_lane; s < p; s += L) {
                 uint32_t idx[2 * NB4];
-                const R F = sample_point<FAM, MIXED, NB4, DC, FIX>(a, cells, c, s, it, nbc, idx);
+                const R F = sample_point<FAM, MIXED, NB4, DC, FIX>(a, cells, c, s, rng, pc, nbc, idx);
                 if (n == 0) {
                     K = F;  // the shift: its own term is zero
                 } else if (n == 1) {
@@ -456,28 +532,18 @@ __device__ __forceinline__ void sample_cubes(const A& a, const typename Prec<MIX
                 }
             }
         }
+        advance();
         if (L == 1u) {
-            if (valid) {
-                // UpdateVariance (Alg. 3): cube mean and the variance of that
-                // mean; at p = 2 (every 1e8-call geometry) S1 = z, S2 = z^2 and
-                // the variance (z^2 - z^2/2)/2 is exactly z^2/4: the z^2 are
-                // summed and the sum scaled once after the loop (exact)
-                RS mean, var;
-                if (p == 2u) {
-                    mean = (RS)K + S1 * RS(0.5);
-                    var = S1 * S1;
-                } else {
-                    mean = (RS)K + S1 * inv_p;
-                    var = (S2 - S1 * S1 * inv_p) * inv_var_den;
-                }
+            if (valid) {  // UpdateVariance (Alg. 3): cube mean and the variance of that mean
+                const RS mean = (RS)K + S1 * inv_p;
+                const RS var = (S2 - S1 * S1 * inv_p) * inv_var_den;
                 if constexpr (sizeof(RS) == 4) {
                     acc.fI.add(mean);
                     acc.fV.add(var);
                     if (a.want_abs) acc.fA.add(fabsf(mean));
                 } else {
                     acc.I += mean;
-                    if (p == 2u) acc.V = fma(S1, S1, acc.V);  // one FMA for the z^2
-                    else acc.V += var;
+                    acc.V += var;
                     if (a.want_abs) acc.A += fabs(mean);
                 }
             }
@@ -491,9 +557,9 @@ __device__ __forceinline__ void sample_cubes(const A& a, const typename Prec<MIX
             double s1 = (double)S1, s2 = (double)S2;
             s2 = fma(dK, fma(cnt, dK, 2.0 * s1), s2);
             s1 = fma(cnt, dK, s1);
-            for (uint32_t off = 1; off < L; off <<= 1) {
-                s1 += __shfl_xor_sync(0xffffffffu, s1, off);
-                s2 += __shfl_xor_sync(0xffffffffu, s2, off);
+            for (uint32_t o = 1; o < L; o <<= 1) {
+                s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+                s2 += __shfl_xor_sync(0xffffffffu, s2, o);
             }
             if (valid && seg_lane == 0) {
                 const double mean = K0 + s1 * a.inv_p;
@@ -502,11 +568,6 @@ __device__ __forceinline__ void sample_cubes(const A& a, const typename Prec<MIX
                 if (a.want_abs) acc.A += fabs(mean);
             }
         }
-    }
-    if (L == 1u && p == 2u) {  // the z^2 / 4 of every cube, scaled once
-        acc.V *= 0.25;
-        acc.fV.hi *= 0.25f;
-        acc.fV.lo *= 0.25f;
     }
 }
 
@@ -521,38 +582,24 @@ __device__ __forceinline__ void sample_cubes(const A& a, const typename Prec<MIX
 template <int FAM, bool MIXED, bool ADJ, int NB4, int DC, bool FIX, class A>
 __device__ __forceinline__ void sample_cube_slice(const A& a, const typename Prec<MIXED>::Cell* cells,
                                                   typename Prec<MIXED>::H* hist, uint64_t cube, uint32_t k,
-                                                  uint32_t split, uint32_t it, uint32_t p,
+                                                  uint32_t split, const SampleRng<NB4>& rng, uint32_t p,
                                                   double (*red)[kVsThreadsMax / 32], double* out)
 {
     using R = typename Prec<MIXED>::R;
     using HT = typename Prec<MIXED>::H;
-    constexpr int DN = 4 * NB4;
-    const uint32_t d = DC ? (uint32_t)DC : a.d, nb = a.nb;
     const uint32_t hist_d = a.hist_d;
     const uint32_t q = (p + split - 1) / split;
     const uint32_t s_lo = k * q, s_hi = min(p, s_lo + q);
     const uint32_t hist_s = (uint32_t)__cvta_generic_to_shared(hist);
     const uint32_t c = (uint32_t)cube;
-    uint32_t nbc[DN];
-    {
-        uint32_t rest = c;
-#pragma unroll
-        for (int j = 0; j < DN; ++j) {
-            if (j < (int)d) {
-                uint32_t qq = __umulhi(rest, a.gmagic);
-                uint32_t r = rest - qq * a.g;
-                if (r >= a.g) { ++qq; r -= a.g; }
-                if (r >= a.g) { ++qq; r -= a.g; }
-                nbc[j] = r * nb;
-                rest = qq;
-            }
-        }
-    }
+    uint32_t nbc[4 * NB4];
+    cube_digits<NB4, DC>(a, c, nbc);
+    const PhiloxCube pc = philox_cube(a, rng.it, c);
     R K = R(0), S1 = R(0), S2 = R(0);
     uint32_t n = 0;
     for (uint32_t s = s_lo + threadIdx.x; s < s_hi; s += blockDim.x) {
         uint32_t idx[2 * NB4];
-        const R F = sample_point<FAM, MIXED, NB4, DC, FIX>(a, cells, c, s, it, nbc, idx);
+        const R F = sample_point<FAM, MIXED, NB4, DC, FIX>(a, cells, c, s, rng, pc, nbc, idx);
         if (n == 0) {
             K = F;  // the shift: its own term is zero
         } else {
@@ -683,11 +730,15 @@ vsample_kernel(const __grid_constant__ VsArgs a)
     using HT = typename Prec<MIXED>::H;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double red[3][kVsThreadsMax / 32];
+    __shared__ uint4 philox_tab[kPhiloxTab * NB4];  // with red at most 960 bytes (mcubes_setup allows 1 KB)
 
     constexpr uint32_t d = D;
     const uint32_t nb = a.nb;
-    Cell* cells = reinterpret_cast<Cell*>(smem);
-    HT* hist = reinterpret_cast<HT*>(smem + cell_bytes(MIXED) * d * nb);
+    // single precision: the histogram first, its address a constant of the
+    // additions (corner8 15.32 -> 14.82 ms per 1e9-call pass with the bins kept
+    // as byte offsets); double precision: the cells first
+    HT* hist = reinterpret_cast<HT*>(smem + (MIXED ? 0u : cell_bytes(false) * d * nb));
+    Cell* cells = reinterpret_cast<Cell*>(smem + (MIXED && ADJ ? hist_smem_bytes(true, a.hist_d * nb) : 0u));
     if constexpr (ADJ) clear_hist(hist, a.hist_d * nb);
     grid_dependency_wait();  // the refinement before this pass (launch_dependent)
     uint32_t it = a.it_fixed;
@@ -700,18 +751,20 @@ vsample_kernel(const __grid_constant__ VsArgs a)
         it = (uint32_t)v.x;
     }
 
+    fill_philox_table<NB4>(philox_tab, a, it);
+    const SampleRng<NB4> rng{it, philox_tab};
     if (a.cells_g) stage_cells<MIXED>(cells, a.cells_g, d, nb);
     else stage_grid<MIXED, FIX>(cells, a.grid, a.grid_lo, a.lo, a.scale, a.cm, d, nb, a.g);
     __syncthreads();
 
     if (a.split > 1) {
         sample_cube_slice<FAM, MIXED, ADJ, NB4, D, FIX>(a, cells, hist, a.cube_begin + blockIdx.x / a.split,
-                                                blockIdx.x % a.split, a.split, it, a.p, red,
+                                                blockIdx.x % a.split, a.split, rng, a.p, red,
                                                 a.part + 3 * (size_t)blockIdx.x);
     } else {
         CubeSums acc;
         sample_cubes<FAM, MIXED, ADJ, NB4, D, FIX>(a, cells, hist, a.cube_begin, a.cube_end - a.cube_begin, a.perm_k, a.perm_inv,
-                                           blockIdx.x, gridDim.x, it, a.lanes, a.p, acc);
+                                           blockIdx.x, gridDim.x, rng, a.lanes, a.p, acc);
         grid_dependents_launch();  // the refinement's blocks may take their places
         block_write_sums<MIXED>(acc, a.want_abs != 0, red, a.part + 3 * (size_t)blockIdx.x);
     }
@@ -758,9 +811,17 @@ inline auto vsample_kernel_ptr(bool mixed, bool adjust, bool fix, int d)
 }
 
 template <int FAM>
-cudaError_t launch_vsample_family(bool mixed, bool adjust, const VsArgs& a, int grid, size_t smem,
+cudaError_t launch_vsample_family(bool mixed, bool adjust, const VsArgs& args, int grid, size_t smem,
                                   cudaStream_t s)
 {
+    VsArgs a = args;
+    const uint64_t n = a.cube_end - a.cube_begin;
+    if (n > 0 && a.split == 1) {  // the cube step of this launch's groups
+        const uint64_t group = (uint64_t)grid * (vsample_threads(FAM, mixed, (int)a.d) / a.lanes);
+        uint64_t m = 1;
+        for (uint32_t j = 0; j < a.d; ++j) m *= a.g;
+        cube_step_digits((group % n) * a.perm_k % n, n, m, a.d, a.g, a.nb, a.cube_step[0], a.cube_step[1]);
+    }
     auto k = vsample_kernel_ptr<FAM>(mixed, adjust, a.fam.fix != 0, (int)a.d);
     cudaError_t e = raise_smem_limit((const void*)k, smem);
     if (e != cudaSuccess) return e;
