@@ -432,9 +432,19 @@ void BatchEngine::live_slots(std::vector<int>* live, ClassMask* class_mask) cons
 // per block, the serving mix without retries at 2000 requests/s p50 2.6 ms and
 // p99 3.9 ms against 15.2 and 21.0; 8192: 3.1 and 4.1 ms, 32768: 7.1 and 8.5).
 constexpr double kMinBlockSamples = 2048.0;
+// A step's chunks, all classes together, fill about kChunkWaves waves of the
+// GPU's resident blocks (three 256-thread blocks per SM); beyond that chunks
+// grow, up to kMaxChunkSamples, so that a block's fixed work (~5 us: staging a
+// segment, writing its histogram) stays small beside its samples.  256
+// requests of 1e5 calls: 20.8 -> 15.6 ms against chunks of 2048 samples
+// (3 waves 16.0, 12 waves 18.1 ms); 1024 integrals of 1e4-1e7 calls, whose
+// chunks would be 2.6e5 samples at 6 waves: 106.6 ms, 105.2 at 12 waves
+// (a finer tail), hence the upper limit.
+constexpr double kChunkWaves = 6.0;
+constexpr double kMaxChunkSamples = 32768.0;
 
 // For every class, lays its live integrals' samples end to end and cuts the
-// line into equal chunks, at least kMinBlockSamples samples each and at most
+// line into equal chunks, at least chunk_min samples each and at most
 // class_blocks(class) of them; cube c of an integral goes to the chunk
 // holding its first sample.  Writes the segment list (class by
 // class, then block by block), every class's block table (a fixed region of
@@ -451,20 +461,24 @@ void BatchEngine::partition(const std::vector<int>& live, int* nseg_out)
     int nseg = 0;
     size_t hist_off = 0;
     size_t j = 0;
+    double all = 0.0;
+    for (int s : live) all += slots_[s].work;
+    const double chunk_min =
+        std::min(std::max(kMinBlockSamples, all / (kChunkWaves * 3.0 * num_sms_)), kMaxChunkSamples);
     while (j < live.size()) {
         const int cls = batch_class(hdesc_[live[j]].family, (int)hdesc_[live[j]].d);
         size_t j1 = j;
         double total = 0.0;
         while (j1 < live.size() && batch_class(hdesc_[live[j1]].family, (int)hdesc_[live[j1]].d) == cls)
             total += slots_[live[j1++]].work;
-        // chunks of at least kMinBlockSamples samples, at most one per block
+        // chunks of at least chunk_min samples, at most one per block
         // of the class's launch (its full occupancy): a step of small
         // requests is cut into few chunks (each block's fixed work -- staging
         // a segment's grid, writing its partial histogram -- stays small
         // beside its samples, and the refinement merges fewer segments), a
         // large batch fills every block
         const int blocks_max = class_blocks(cls);
-        const int blocks = (int)std::max(1.0, std::min((double)blocks_max, std::ceil(total / kMinBlockSamples)));
+        const int blocks = (int)std::max(1.0, std::min((double)blocks_max, std::ceil(total / chunk_min)));
         class_load_[cls] = total * (4.0 + hdesc_[live[j]].d) / blocks;
         uint32_t* blk_seg = table + (size_t)cls * (bmax_ + 1);
         const double chunk = total / blocks;
@@ -536,6 +550,10 @@ BatchArgs BatchEngine::sample_args(int cls) const
     a.blk_seg = (const uint32_t*)blk_seg_.ptr + (size_t)cls * (bmax_ + 1);
     a.seg_part = (double*)seg_part_.ptr;
     a.seg_hist = seg_hist_.ptr;
+    a.cells = cells_.ptr;
+    a.cell_stride = cell_bytes(mixed_) * (size_t)kDMax * opts_.nbins;
+    a.nb = (uint32_t)opts_.nbins;
+    a.pad = 0;
     return a;
 }
 

@@ -16,6 +16,14 @@
 
 namespace mc {
 
+// A value that every lane of the warp holds, moved to a uniform register (the
+// result of a warp reduction is one): operands and round keys that are launch
+// constants in the single-integral kernels are segment constants here (64
+// integrals of 2e6 calls: corner d = 8 6.60 -> 6.39, osc d = 10 8.22 -> 7.97
+// cycles per SM and sample against reading them from shared memory).
+__device__ __forceinline__ uint32_t uni(uint32_t v) { return __reduce_or_sync(0xffffffffu, v); }
+__device__ __forceinline__ float uni(float v) { return __uint_as_float(uni(__float_as_uint(v))); }
+
 // One kernel per (family, dimension D): every segment it samples belongs to
 // an integral of that dimension.  Registers are bounded as for the
 // single-integral kernel of the same family and axis count (3 or 4 resident
@@ -41,30 +49,38 @@ vsample_batch_kernel(const __grid_constant__ BatchArgs a)
     for (uint32_t si = s_begin; si < s_end; ++si) {
         const BatchSeg seg = a.segs[si];
         __syncthreads();  // the previous segment is done with sd, cells and hist
+        // the integral's state, descriptor and map cells together (their places
+        // follow from the slot): one trip to memory
+        const BatchState& B = a.st[seg.slot];
+        const int2 now = ld_volatile_int2(&B.it);
         {
             const uint32_t* src = reinterpret_cast<const uint32_t*>(a.desc + seg.slot);
             uint32_t* dst = reinterpret_cast<uint32_t*>(&sd);
             for (uint32_t i = threadIdx.x; i < sizeof(BatchDesc) / 4; i += blockDim.x) dst[i] = src[i];
         }
+        HT* hist = reinterpret_cast<HT*>(smem + (MIXED ? 0u : cell_bytes(false) * D * a.nb));
+        Cell* cells = reinterpret_cast<Cell*>(smem + (MIXED ? hist_smem_bytes(true, D * a.nb) : 0u));
+        if (seg.adjust) clear_hist(hist, D * a.nb);
+        stage_cells<MIXED>(cells, static_cast<const unsigned char*>(a.cells) + a.cell_stride * seg.slot, D, a.nb);
         __syncthreads();
         // an integral that finished in an earlier iteration of this step (a
         // step may run several) is skipped; only the refinement changes the state
-        const BatchState& B = a.st[seg.slot];
-        if (B.done || (int)B.it >= sd.itmax) continue;
+        if (now.y || now.x >= sd.itmax) continue;
         // this iteration adjusts while it < ita (a step's iterations may cross
         // ita); the refinement reads the flag back
-        const bool adjust = seg.adjust && (int)B.it < sd.ita;
+        const bool adjust = seg.adjust && now.x < sd.ita;
         if (threadIdx.x == 0) a.segs[si].adjust = adjust ? 1u : 0u;
         constexpr uint32_t d = D;
-        const uint32_t nb = sd.nb;
-        HT* hist = reinterpret_cast<HT*>(smem + (MIXED ? 0u : cell_bytes(false) * d * nb));
-        Cell* cells = reinterpret_cast<Cell*>(smem + (MIXED ? hist_smem_bytes(true, d * nb) : 0u));
-        if (adjust) clear_hist(hist, d * nb);
-        stage_cells<MIXED>(cells, sd.cells, d, nb);
-        const BatchView v{d,        nb,           sd.g,     sd.gmagic,         sd.key0,          sd.key1, d,
-                          sd.jac0,  sd.phi_scale_f, sd.inv_p, sd.inv_var_den, sd.inv_p_f, sd.inv_var_den_f, 0u,
-                          cube_step, sd.fam};
-        const uint32_t it = B.it;
+        const uint32_t nb = a.nb;
+        FamParams uf;  // single precision: the integrand's constants (those it reads)
+        if constexpr (MIXED) {
+#pragma unroll
+            for (int i = 0; i < kParMax; ++i) uf.cf[i] = uni(sd.fam.cf[i]);
+        }
+        const BatchView v{d,        nb,           uni(sd.g), uni(sd.gmagic),   uni(sd.key0),     uni(sd.key1), d,
+                          sd.jac0,  uni(sd.phi_scale_f), sd.inv_p, sd.inv_var_den, sd.inv_p_f, sd.inv_var_den_f, 0u,
+                          cube_step, MIXED ? uf : sd.fam};
+        const uint32_t it = (uint32_t)now.x;
         fill_philox_table<NB4>(philox_tab, v, it);
         const SampleRng<NB4> rng{it, philox_tab};
         if (threadIdx.x == blockDim.x - 1) {

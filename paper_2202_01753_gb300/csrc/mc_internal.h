@@ -169,7 +169,7 @@ struct BatchDesc {
 };
 
 // Per-integral iteration state of a batch (device).
-struct BatchState {
+struct alignas(8) BatchState {
     uint32_t it;
     int done, error, n, converged, pad;
     double estimate, sigma, chi2_dof;
@@ -192,6 +192,9 @@ struct BatchArgs {
     const uint32_t* blk_seg;    // block b samples segments [blk_seg[b], blk_seg[b+1]) (this class's table)
     double* seg_part;           // [segment][3] partial sums
     void* seg_hist;             // partial histograms (float in mixed, double in fp64)
+    const void* cells;          // slot s's map cells at cells + s * cell_stride bytes
+    uint64_t cell_stride;
+    uint32_t nb, pad;           // bins per axis, the same for every slot
 };
 
 struct BatchRefineArgs {
