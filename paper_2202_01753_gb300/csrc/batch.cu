@@ -145,6 +145,7 @@ __device__ void refine_one(const BatchRefineArgs& a, uint32_t j, RebinShared& sh
             sh.Blo[k] = grid_lo[k];
             D.hist[off + k] = acc;
         }
+        load_log_tables(sh);
         if (!rebin_block(sh, nb, a.alpha, &st->error, &st->done)) return;
         const double inv_g = 1.0 / (double)D.g;
         for (int k = threadIdx.x; k < nb; k += kRefineThreads) {

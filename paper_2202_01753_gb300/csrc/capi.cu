@@ -314,6 +314,34 @@ void philox_round_keys(uint64_t seed, uint32_t rk[10][2])
 
 }  // namespace mc
 
+namespace mc {
+// How many threads share a cube.  Single precision: enough cube-lanes to cover
+// the resident threads several times, and a bounded number of samples per
+// lane.  Double precision: the least rounds x (samples per lane + merge), where
+// a merge of L lanes takes about 10 + 2 log2 L FP64 warp instructions of 16
+// cycles beside a sample's ~320 (f2 d = 6 at 1e6 calls, 3 samples in each of
+// 2.6e5 cubes: 2 lanes 60.6 us per pass, 1 lane 45.5; gauss d = 2 at 1e6, 5e5
+// cubes of 2: 49.7 and 31.4).
+int choose_lanes(bool mixed, long long m, long long p, long long resident)
+{
+    int L = 1;
+    if (mixed) {
+        while (L < 32 && 2 * L <= p && (m * L < 4 * resident || p / L > 64)) L *= 2;
+        return L;
+    }
+    double best = 0.0;
+    for (int l = 1, lg = 0; l <= 32 && (l == 1 || l <= p); l *= 2, ++lg) {
+        const double rounds = (double)((m * l + resident - 1) / resident);
+        const double cost = rounds * ((double)((p + l - 1) / l) + (l > 1 ? 0.5 + 0.1 * lg : 0.0));
+        if (l == 1 || cost < best) {
+            best = cost;
+            L = l;
+        }
+    }
+    return L;
+}
+}  // namespace mc
+
 static mcubes_status cuda_fail(mcubes_ctx* c, cudaError_t e)
 {
     if (c) std::snprintf(c->cuda_err, sizeof c->cuda_err, "%s: %s", cudaGetErrorName(e), cudaGetErrorString(e));
@@ -481,15 +509,6 @@ mcubes_status mcubes_destroy(mcubes_ctx* c)
     return MCUBES_OK;
 }
 
-// Chooses how many threads share a cube: enough cube-lanes to cover the
-// resident threads several times, and a bounded number of samples per lane.
-static int choose_lanes(long long m, long long p, long long resident)
-{
-    int L = 1;
-    while (L < 32 && 2 * L <= p && (m * L < 4 * resident || p / L > 64)) L *= 2;
-    return L;
-}
-
 mcubes_status mcubes_setup(mcubes_ctx* c, int id, const double* params, int nparams, int d,
                            const double* lo, const double* hi, long long ncall, int itmax,
                            double rel_tol, double abs_tol)
@@ -554,13 +573,15 @@ mcubes_status mcubes_setup(mcubes_ctx* c, int id, const double* params, int npar
     c->grid_res_noadj = c->grid_noadj;
     const int threads = vsample_threads(id, c->mixed, d);
     const long long resident = (long long)std::max(occ_adj, occ_noadj) * c->num_sms * threads;
-    c->lanes = c->opts.lanes_per_cube > 0 ? c->opts.lanes_per_cube : choose_lanes(m, p, resident);
+    c->lanes = c->opts.lanes_per_cube > 0 ? c->opts.lanes_per_cube : choose_lanes(c->mixed, m, p, resident);
     // Cube-split mode: when the cubes cannot keep a quarter of the resident
     // threads busy (few cubes with many samples each), several blocks share
-    // one cube, so that about two waves of blocks sample every iteration.
+    // one cube, so that one wave of blocks samples every iteration (gauss3, 64
+    // cubes of 16384 samples: 47.0 us per pass against 53.7 with two waves, and
+    // half as many slices for the refinement to merge, 14.0 us against 18.6).
     c->split = 1;
     if (c->opts.lanes_per_cube == 0 && m * c->lanes * 4 < resident && p >= 2 * threads) {
-        const long long want = (2LL * std::max(c->grid_adj, c->grid_noadj) + m - 1) / m;
+        const long long want = std::max(c->grid_adj, c->grid_noadj) / m;
         c->split = (int)std::max(1LL, std::min(want, p / threads));
         if (c->split > 1) c->grid_adj = c->grid_noadj = (int)(m * c->split);
     }

@@ -87,17 +87,19 @@ __device__ __forceinline__ LogPair ld_pair(const LogPair* p)
 // the table point at or below m, r = (m - c_j)/c_j in [0, 2^-8), d_k =
 // 1 + k/65536 the second table point at or below 1 + r and r2 = (r - k/65536)/d_k
 // in [0, 2^-16): every quantity is non-negative.
-// The mantissa's part, from its 52 fraction bits f: ln m in Q64 (< ln 2).
-__device__ __forceinline__ uint64_t fx_ln_mantissa(uint64_t f)
+// The mantissa's part, from its 52 fraction bits f: ln m in Q64 (< ln 2);
+// load(t, i): entry i of table t (0: c_j, 1: d_k).
+template <class Load>
+__device__ __forceinline__ uint64_t fx_ln_mantissa_t(uint64_t f, Load load)
 {
     const int j = (int)(f >> 44);
     // m - c_j is the mantissa's low 44 bits (Q52); r = (m - c_j)/c_j in Q64 (< 2^56)
-    const LogPair cj = ld_pair(&kLogC[j]);
+    const LogPair cj = load(0, j);
     const uint64_t r = __umul64hi((f & 0xFFFFFFFFFFFull) << 13, cj.inv);
     // second step: k = the top 8 bits of r (r < 2^-8), r - k/65536 its low 48 bits
     // (Q64); r2 = (r - k/65536)/d_k in Q64 (< 2^48)
     const int k = (int)(r >> 48);
-    const LogPair dk = ld_pair(&kLogD[k]);
+    const LogPair dk = load(1, k);
     const uint64_t R = __umul64hi((r & 0xFFFFFFFFFFFFull) << 16, dk.inv) >> 15;
     // ln(1 + r2) = r2 - r2^2/2 + r2^3/3 (+ r2^4/4 < 2^-66).  r2^2 from the top 32
     // bits of r2 (H = r2 in Q48; the dropped low bits move it by < 2^-62) and
@@ -107,6 +109,11 @@ __device__ __forceinline__ uint64_t fx_ln_mantissa(uint64_t f)
     const uint32_t cube = (uint32_t)(((uint64_t)(uint32_t)sq * H) >> 48);  // r2^3, Q64 (< 2^16)
     const uint64_t l2 = R - (sq >> 1) + __umulhi(cube, q32_inv(3));        // ln(1 + r2), Q64
     return cj.ln + dk.ln + l2;
+}
+
+__device__ __forceinline__ uint64_t fx_ln_mantissa(uint64_t f)
+{
+    return fx_ln_mantissa_t(f, [](int t, int i) { return ld_pair(t ? &kLogD[i] : &kLogC[i]); });
 }
 
 __device__ __forceinline__ double fx_log(double x)

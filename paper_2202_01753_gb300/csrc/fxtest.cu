@@ -43,6 +43,7 @@ rebin_kernel(int nb, double alpha, double* C, double* B, double* Blo)
         s.B[k] = B[k];
         s.Blo[k] = Blo[k];
     }
+    mc::refine_detail::load_log_tables(s);
     if (!mc::refine_detail::rebin_block(s, nb, alpha, &g_rebin_flags[0], &g_rebin_flags[1])) return;
     for (int k = threadIdx.x; k < nb; k += mc::kRefineThreads) {
         B[k] = s.B[k];

@@ -10,6 +10,31 @@
 
 namespace mc {
 
+namespace fx {
+// Reads the tables of an FP64 family's functions once, a load per 128-byte
+// line, so that the samples' dependent lookups find them in L1 (called before
+// the launch's wait, when the SM is idle).
+__device__ __forceinline__ void warm_lines(const void* p, uint32_t bytes)
+{
+    if (threadIdx.x < bytes / 128u) {
+        const uint32_t v = __ldg(static_cast<const uint32_t*>(p) + threadIdx.x * 32u);
+        asm volatile("" ::"r"(v));
+    }
+}
+template <int FAM> __device__ __forceinline__ void warm_tables()
+{
+    if constexpr (FAM == MCUBES_F_GAUSS || FAM == MCUBES_F_C0 || FAM == MCUBES_F_DISCONT || FAM == MCUBES_F_COSMO6) {
+        warm_lines(kExpK16, sizeof kExpK16);
+        warm_lines(kExp2, sizeof kExp2);
+    }
+    if constexpr (FAM == MCUBES_F_COSMO6) {
+        warm_lines(kLogC, sizeof kLogC);
+        warm_lines(kLogD, sizeof kLogD);
+    }
+    if constexpr (FAM == MCUBES_F_OSC) warm_lines(kCosSin, sizeof kCosSin);
+}
+}  // namespace fx
+
 // Programmatic dependent launch (launch_dependent): a kernel's blocks may be
 // placed, and run up to their wait, once every block of the kernel before it
 // in the stream has called grid_dependents_launch or ended; the wait ends when

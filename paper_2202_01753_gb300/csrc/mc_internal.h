@@ -282,6 +282,7 @@ cudaError_t vsample_occupancy(int family, bool mixed, bool adjust, bool fix, int
 // *jac0 untouched where it does not.
 void affine_prepare(int id, const double* params, int d, const double* lo, const double* scale, long long g, int nb,
                     FamParams* fp, CellMap* cm, double* jac0);
+int choose_lanes(bool mixed, long long m, long long p, long long resident);  // threads per cube
 uint64_t cube_permutation(uint64_t n);
 template <class T> void set_cube_order(T& a, uint64_t n)  // of a range of n cubes
 {

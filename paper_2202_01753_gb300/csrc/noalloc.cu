@@ -131,10 +131,8 @@ extern "C" mcubes_status mcubes_sample_range_noalloc(
         // kMaxBlocks here), so the cubes' sums are grouped into other block
         // partials: results agree with mcubes_sample_range to rounding, not
         // bit for bit.
-        int lanes = 1;
         const long long resident = (long long)std::max(occ, occ_other) * sms * vsample_threads(integrand_id, mixed, d);
-        while (lanes < 32 && 2 * lanes <= p && (m * lanes < 4 * resident || p / lanes > 64)) lanes *= 2;
-        a.lanes = (uint32_t)lanes;
+        a.lanes = (uint32_t)choose_lanes(mixed, m, p, resident);
         a.hist_d = (uint32_t)d;
         a.split = 1;
         a.cube_begin = (uint64_t)cube_begin;

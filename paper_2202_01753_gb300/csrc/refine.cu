@@ -14,15 +14,18 @@ using namespace refine_detail;
 
 // Adjust-Bin-Bounds of axis ax (rebin_block): the row of the pass's histogram
 // is read and cleared, the new edges and map cells written (in m-Cubes1D for
-// every axis).
-// The edges are read before the sampling pass has ended: nothing writes them
-// between two refinements.
+// every axis).  The tables and edges are read before the sampling pass has
+// ended: nothing writes them between two refinements.  (Sharing an axis's
+// edges and cells among a cluster of two or four blocks measured no faster,
+// f5 d = 8 at 1e5 calls 8% slower: the cluster's blocks have to find room
+// beside the sampling blocks.)
 static __device__ __forceinline__ void rebin_axis(const RefineArgs& a, int ax)
 {
     __shared__ RebinShared s;
     const int nb = a.nb;
     const size_t off = (size_t)ax * nb;
     const int rows = a.hist_d == a.d ? 1 : a.d;  // m-Cubes1D: axis 0's edges go to every axis
+    load_log_tables(s);
     for (int k = threadIdx.x; k < nb; k += kRefineThreads) {
         s.B[k] = a.grid[off + k];
         s.Blo[k] = a.grid_lo[off + k];

@@ -161,7 +161,10 @@ static __device__ void finalize_iteration(const double* part, int nparts, double
         // partials loaded ahead at a time; then the cube's mean and the variance
         // of that mean (UpdateVariance of Alg. 3) with the reciprocals formed once
         const int ncubes = nparts / split;
+        // samples of a slice: q in the first k_full, then the rest, then none
         const double q = ceil(p / split);
+        const int k_full = (int)(p / q);
+        const double rest = p - q * k_full;
         const double inv_p = 1.0 / p, inv_var_den = inv_p / (p - 1.0);
         for (int cb = threadIdx.x; cb < ncubes; cb += kRedThreads) {
             const double* v = part + 3 * (size_t)cb * split;
@@ -180,7 +183,7 @@ static __device__ void finalize_iteration(const double* part, int nparts, double
                 for (int u = 0; u < 8; ++u) {
                     const int k = k0 + u;
                     if (k < split) {
-                        const double nk = fmin(q, fmax(p - q * k, 0.0));
+                        const double nk = k < k_full ? q : (k == k_full ? rest : 0.0);
                         const double dK = a0[u] - K0;
                         S2 += fma(dK, fma(nk, dK, 2.0 * a1[u]), a2[u]);
                         S1 += fma(nk, dK, a1[u]);
@@ -336,7 +339,8 @@ static __device__ __noinline__ u128 power_weight(double q, double alpha)
 // fixed-point reciprocal, and for alpha = 3/2 a fixed-point square root.  The
 // FP64 form of this (two divisions, a logarithm's rounding, a root) was ~75
 // dependent FP64 instructions, 66 cycles each.
-static __device__ __forceinline__ u128 compressed_weight(double sm3, const IntProd& inv_total, double alpha)
+static __device__ __forceinline__ u128 compressed_weight(double sm3, const IntProd& inv_total, double alpha,
+                                                         const fx::LogPair (*logs)[256])
 {
     if (!(sm3 > 0.0)) return 0;
     IntProd r = int_prod_mul2(int_prod_of(sm3), inv_total);
@@ -349,7 +353,7 @@ static __device__ __forceinline__ u128 compressed_weight(double sm3, const IntPr
     }
     if (r.e >= 0) return (u128)1 << 100;                  // r >= 1
     // |ln r| = -e ln 2 - ln m as a 128-bit Q64 magnitude
-    const uint64_t U = fx::fx_ln_mantissa((r.m >> 11) & 0xFFFFFFFFFFFFFull);
+    const uint64_t U = fx::fx_ln_mantissa_t((r.m >> 11) & 0xFFFFFFFFFFFFFull, [&](int t, int i) { return logs[t][i]; });
     const u128 ln = (u128)(uint32_t)(-r.e) * fx::kLn2Q64 - U;
     const int z = clz_u128(ln);
     const IntProd L{(uint64_t)((ln << z) >> 64), 63 - z};
@@ -402,10 +406,20 @@ struct RebinShared {
     u128 X[kNbMax];                 // nb x the inclusive cumulative compressed weights, Q100
     u128 wtot[kWarps];
     u128 W[kPerThread];             // weight up to each round's last bin
+    fx::LogPair logs[2][256];       // the logarithm's tables (load_log_tables)
     uint32_t emax[kWarps];
     uint32_t sum[3][kWarps];
     long long ends[4];              // C_0, C_1, C_{nb-2}, C_{nb-1} in the fixed-point scale
 };
+
+// The logarithm's tables into shared memory: a bin's two lookups depend on each
+// other, ~700 cycles each from a cold cache.
+static __device__ __forceinline__ void load_log_tables(RebinShared& s)
+{
+    const int t = threadIdx.x;
+    static_assert(kRefineThreads == 512, "one entry per thread");
+    s.logs[t >> 8][t & 255] = fx::ld_pair(t >= 256 ? &fx::kLogD[t & 255] : &fx::kLogC[t & 255]);
+}
 
 // Adjust-Bin-Bounds of one axis (Lepage 1978, as the paper's Alg. 2 cites):
 // smooth the bin sums with their neighbours, normalise, compress with
@@ -422,10 +436,10 @@ struct RebinShared {
 // cycles per step, so one block per axis is enough (the FP64 form took
 // 27,500 cycles spread over a cluster of four blocks per axis, five cluster
 // barriers included; refine.cu has both sides' times).
-// On entry s.C, s.B and s.Blo hold the histogram and the edges (written by
-// this block, no barrier needed); true: s.B and s.Blo hold the new edges.
-// False: the grid stays (no information on the axis, or a non-finite sum,
-// which is reported in *error and *done).
+// On entry s.C, s.B, s.Blo and s.logs hold the histogram, the edges and the
+// logarithm's tables (written by this block, no barrier needed); true: s.B and
+// s.Blo hold the new edges.  False: the grid stays (no information on the axis,
+// or a non-finite sum, which is reported in *error and *done).
 static __device__ bool rebin_block(RebinShared& s, int nb, double alpha, int* error, int* done)
 {
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -494,7 +508,7 @@ static __device__ bool rebin_block(RebinShared& s, int nb, double alpha, int* er
 #pragma unroll 1
     for (int i = 0; i * kRefineThreads < nb; ++i) {
         const int k = t + i * kRefineThreads;
-        const u128 w = k < nb ? compressed_weight(smoothed3(s.C, k, nb), inv_total, alpha) : (u128)0;
+        const u128 w = k < nb ? compressed_weight(smoothed3(s.C, k, nb), inv_total, alpha, s.logs) : (u128)0;
         const u128 c = u128_scan(w, W, s.wtot, &s.W[i]);
         if (k < nb) s.X[k] = (u128)(uint32_t)nb * c;
         __syncthreads();

@@ -740,6 +740,7 @@ vsample_kernel(const __grid_constant__ VsArgs a)
     HT* hist = reinterpret_cast<HT*>(smem + (MIXED ? 0u : cell_bytes(false) * d * nb));
     Cell* cells = reinterpret_cast<Cell*>(smem + (MIXED && ADJ ? hist_smem_bytes(true, a.hist_d * nb) : 0u));
     if constexpr (ADJ) clear_hist(hist, a.hist_d * nb);
+    if constexpr (!MIXED) fx::warm_tables<FAM>();
     grid_dependency_wait();  // the refinement before this pass (launch_dependent)
     uint32_t it = a.it_fixed;
     if (a.st != nullptr) {
@@ -769,7 +770,7 @@ vsample_kernel(const __grid_constant__ VsArgs a)
         block_write_sums<MIXED>(acc, a.want_abs != 0, red, a.part + 3 * (size_t)blockIdx.x);
     }
     if constexpr (ADJ) {
-        __syncthreads();
+        // (every warp has passed a barrier since its last histogram addition)
         // the block's histogram goes into the pass's accumulator once: one
         // global reduction per non-empty bin (no per-sample global atomics)
         for (uint32_t i = threadIdx.x; i < a.hist_d * nb; i += blockDim.x) {
