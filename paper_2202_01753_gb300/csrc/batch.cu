@@ -393,10 +393,15 @@ cudaError_t BatchEngine::flush_admissions()
 {
     if (pending_.empty()) return cudaSuccess;
     cudaError_t e;
-    for (int slot : pending_) {
-        if ((e = cudaMemcpyAsync((BatchDesc*)desc_.ptr + slot, &hdesc_[slot], sizeof(BatchDesc),
+    // runs of neighbouring slots in one copy each (a batch's slots are one run)
+    std::sort(pending_.begin(), pending_.end());
+    for (size_t i = 0; i < pending_.size();) {
+        size_t k = i + 1;
+        while (k < pending_.size() && pending_[k] == pending_[k - 1] + 1) ++k;
+        if ((e = cudaMemcpyAsync((BatchDesc*)desc_.ptr + pending_[i], &hdesc_[pending_[i]], sizeof(BatchDesc) * (k - i),
                                  cudaMemcpyHostToDevice, stream_)))
             return e;
+        i = k;
     }
     uint32_t* hs = h_small_;  // staging: slot list
     for (size_t i = 0; i < pending_.size(); ++i) hs[i] = (uint32_t)pending_[i];

@@ -497,6 +497,7 @@ mcubes_status mcubes_destroy(mcubes_ctx* c)
     c->cells.release();
     c->state.release();
     c->range_out.release();
+    if (c->stage) cudaFreeHost(c->stage);
     delete c->engine;
     c->engine = nullptr;
     recycle_events(c);
@@ -560,8 +561,8 @@ mcubes_status mcubes_setup(mcubes_ctx* c, int id, const double* params, int npar
     const size_t on_chip = (size_t)d * nb * cell_bytes(c->mixed) + (size_t)c->hist_d * nb * hist_bytes(c->mixed);
     if (on_chip + 1024 > (size_t)smem_limit) return MCUBES_EINVAL;
     int occ_adj = 0, occ_noadj = 0;
-    MC_CHECK(c, vsample_occupancy(id, c->mixed, true, fp.fix != 0, d, c->smem_adj, &occ_adj));
-    MC_CHECK(c, vsample_occupancy(id, c->mixed, false, fp.fix != 0, d, c->smem_noadj, &occ_noadj));
+    MC_CHECK(c, c->occupancy(id, true, fp.fix != 0, c->smem_adj, &occ_adj));
+    MC_CHECK(c, c->occupancy(id, false, fp.fix != 0, c->smem_noadj, &occ_noadj));
     if (occ_adj < 1 || occ_noadj < 1) return MCUBES_EINVAL;
     if (c->opts.blocks_per_sm > 0) {
         occ_adj = std::min(occ_adj, c->opts.blocks_per_sm);
@@ -661,17 +662,22 @@ mcubes_status mcubes_setup(mcubes_ctx* c, int id, const double* params, int npar
     r.alpha = c->opts.alpha;
     r.m = (double)m;
 
-    // initial state: uniform grid, empty history
-    DevState hst;
-    std::memset(&hst, 0, offsetof(DevState, hist_I));
-    hst.rel_tol = rel_tol;
-    hst.abs_tol = abs_tol;
-    MC_CHECK(c, cudaMemcpyAsync(c->state.ptr, &hst, offsetof(DevState, hist_I), cudaMemcpyHostToDevice, c->stream));
-    MC_CHECK(c, launch_init_grid((double*)c->grid.ptr, (double*)c->grid.ptr + (size_t)d * nb, d, nb, c->stream));
-    MC_CHECK(c, ctx_refresh_cells(c));
-    MC_CHECK(c, cudaMemsetAsync(c->hist.ptr, 0, sizeof(double) * d * nb, c->stream));
-    MC_CHECK(c, cudaMemsetAsync(c->hist_acc.ptr, 0, sizeof(double) * c->hist_d * nb, c->stream));
-    MC_CHECK(c, cudaStreamSynchronize(c->stream));  // hst lives on this stack frame
+    // initial state: uniform grid and its cells, empty histograms and history
+    SetupArgs sa;
+    std::memset(&sa, 0, sizeof sa);
+    sa.grid = r.grid;
+    sa.grid_lo = r.grid_lo;
+    sa.hist = r.hist;
+    sa.hist_acc = r.hist_acc;
+    sa.cells = c->cells.ptr;
+    sa.st = r.st;
+    sa.box = c->cellbox;
+    sa.rel_tol = rel_tol;
+    sa.abs_tol = abs_tol;
+    sa.d = d;
+    sa.nb = nb;
+    sa.hist_d = c->hist_d;
+    MC_CHECK(c, launch_setup(sa, c->stream));
     c->prob_params.assign(params, params + std::max(nparams, 0));
     c->prob_lo.assign(lo, lo + d);
     c->prob_hi.assign(hi, hi + d);
@@ -724,9 +730,10 @@ mcubes_status mcubes_result_get(mcubes_ctx* c, mcubes_result* out)
     if (!c || !out) return MCUBES_EINVAL;
     if (!c->ready) return MCUBES_ESTATE;
     MC_CHECK(c, cudaSetDevice(c->device));
-    DevState h;
-    MC_CHECK(c, cudaMemcpyAsync(&h, c->state.ptr, offsetof(DevState, hist_I), cudaMemcpyDeviceToHost, c->stream));
+    MC_CHECK(c, c->stage_reserve());
+    MC_CHECK(c, cudaMemcpyAsync(c->stage, c->state.ptr, offsetof(DevState, hist_I), cudaMemcpyDeviceToHost, c->stream));
     MC_CHECK(c, cudaStreamSynchronize(c->stream));
+    const DevState& h = *static_cast<const DevState*>(c->stage);  // its part before the history
     out->estimate = h.estimate;
     out->sigma = h.sigma;
     out->chi2_dof = h.chi2_dof;
@@ -758,17 +765,19 @@ mcubes_status mcubes_trace_get(mcubes_ctx* c, double* I_it, double* var_it, int 
     if (!c || cap < 0) return MCUBES_EINVAL;
     if (!c->ready) return MCUBES_ESTATE;
     MC_CHECK(c, cudaSetDevice(c->device));
-    int hn = 0;
-    MC_CHECK(c, cudaMemcpyAsync(&hn, (char*)c->state.ptr + offsetof(DevState, n), sizeof(int),
+    // the count and as much of both histories as can have been recorded, one wait
+    const int most = std::min(cap, c->itmax);
+    MC_CHECK(c, c->stage_reserve());
+    DevState& h = *static_cast<DevState*>(c->stage);
+    MC_CHECK(c, cudaMemcpyAsync(&h, c->state.ptr, offsetof(DevState, hist_I) + sizeof(double) * most,
                                 cudaMemcpyDeviceToHost, c->stream));
+    if (most > 0 && var_it)
+        MC_CHECK(c, cudaMemcpyAsync(h.hist_V, (char*)c->state.ptr + offsetof(DevState, hist_V), sizeof(double) * most,
+                                    cudaMemcpyDeviceToHost, c->stream));
     MC_CHECK(c, cudaStreamSynchronize(c->stream));
-    const int k = std::min(hn, cap);
-    if (k > 0 && I_it)
-        MC_CHECK(c, cudaMemcpy(I_it, (char*)c->state.ptr + offsetof(DevState, hist_I), sizeof(double) * k,
-                               cudaMemcpyDeviceToHost));
-    if (k > 0 && var_it)
-        MC_CHECK(c, cudaMemcpy(var_it, (char*)c->state.ptr + offsetof(DevState, hist_V), sizeof(double) * k,
-                               cudaMemcpyDeviceToHost));
+    const int hn = h.n, k = std::min(hn, most);
+    if (k > 0 && I_it) std::memcpy(I_it, h.hist_I, sizeof(double) * k);
+    if (k > 0 && var_it) std::memcpy(var_it, h.hist_V, sizeof(double) * k);
     if (n) *n = hn;
     return MCUBES_OK;
 }

@@ -59,6 +59,41 @@ struct mcubes_ctx {
     std::vector<int> batch_slots;       // engine slot of each request of the last mcubes_integrate_batch
     std::vector<int> batch_dims;        // and its dimension
 
+    // pinned landing place of the state read-backs (a pageable one costs a copy
+    // and a wait of its own each)
+    void* stage = nullptr;
+    cudaError_t stage_reserve()
+    {
+        return stage ? cudaSuccess : cudaHostAlloc(&stage, sizeof(mc::DevState), cudaHostAllocDefault);
+    }
+
+    // Resident blocks per SM of the kernel and shared-memory size asked for
+    // last, adjusting and not: a program that integrates again with the same
+    // shape does not ask the driver again.
+    struct Occ {
+        int id = -1, d = 0, blocks = 0;
+        bool mixed = false, fix = false;
+        size_t smem = 0;
+    } occ[2];
+    cudaError_t occupancy(int id, bool adjust, bool fix, size_t smem, int* blocks)
+    {
+        Occ& o = occ[adjust ? 1 : 0];
+        if (o.id != id || o.d != d || o.mixed != mixed || o.fix != fix || o.smem != smem) {
+            const cudaError_t e = mc::vsample_occupancy(id, mixed, adjust, fix, d, smem, &o.blocks);
+            if (e != cudaSuccess) {
+                o.id = -1;
+                return e;
+            }
+            o.id = id;
+            o.d = d;
+            o.mixed = mixed;
+            o.fix = fix;
+            o.smem = smem;
+        }
+        *blocks = o.blocks;
+        return cudaSuccess;
+    }
+
     bool timing = false;
     std::vector<mc::EventPair> ev_sample, ev_refine;
     size_t n_sample = 0, n_refine = 0;

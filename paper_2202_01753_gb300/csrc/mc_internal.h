@@ -327,7 +327,18 @@ template <class T> void set_moment_scales(T& a, long long p)
 cudaError_t launch_refine(const RefineArgs& a, cudaStream_t s);
 cudaError_t launch_reduce_range(const double* part, double* hist_acc, int nblocks, int d, int nb, int adjust,
                                 double* out_sums, double* out_hist, cudaStream_t s);
-cudaError_t launch_init_grid(double* grid, double* grid_lo, int d, int nb, cudaStream_t s);
+struct SetupArgs {
+    double* grid;       // [d][nb] edge high parts
+    double* grid_lo;    // [d][nb] low parts
+    double* hist;       // [d][nb]
+    double* hist_acc;   // [hist_d][nb]
+    void* cells;        // [d][nb] map cells
+    DevState* st;
+    CellBox box;
+    double rel_tol, abs_tol;
+    int d, nb, hist_d;
+};
+cudaError_t launch_setup(const SetupArgs& a, cudaStream_t s);
 // Sums nranks partials ([nranks][len], rank order) element by element in rank
 // order: the first MCUBES_SHARD_HEAD sums go to part[0..], the rest to hist.
 cudaError_t launch_combine_shards(const double* gathered, int nranks, int len, double* part, double* hist,

@@ -119,7 +119,15 @@ __global__ void combine_shards_kernel(const double* gathered, int nranks, int le
     else hist[i - MCUBES_SHARD_HEAD] = s;
 }
 
-// Map cells of the whole grid (set-up, and after the grid is replaced).
+// Map cell i (axis j) of a context's grid.
+__device__ __forceinline__ void write_cell(const CellBox& box, int j, int i, DD left, DD right, int nb, void* out)
+{
+    if (box.mixed) static_cast<float2*>(out)[i] = map_cell_f32(left, right, box.lo[j], box.scale[j], nb);
+    else if (box.cm.fbits) static_cast<double2*>(out)[i] = map_cell_fix(left, right, box.cm, j);
+    else static_cast<double2*>(out)[i] = map_cell_f64(left, right, box.lo[j], box.scale[j], 1.0 / (double)box.g);
+}
+
+// Map cells of the whole grid (after the grid is replaced).
 __global__ void cells_kernel(const double* grid, const double* grid_lo, const __grid_constant__ CellBox box, int d, int nb, void* out)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -127,27 +135,41 @@ __global__ void cells_kernel(const double* grid, const double* grid_lo, const __
     const int j = i / nb, k = i - j * nb;
     const DD right = edge_right(grid + (size_t)j * nb, grid_lo + (size_t)j * nb, k);
     const DD left = edge_left(grid + (size_t)j * nb, grid_lo + (size_t)j * nb, k);
-    if (box.mixed) static_cast<float2*>(out)[i] = map_cell_f32(left, right, box.lo[j], box.scale[j], nb);
-    else if (box.cm.fbits) static_cast<double2*>(out)[i] = map_cell_fix(left, right, box.cm, j);
-    else static_cast<double2*>(out)[i] = map_cell_f64(left, right, box.lo[j], box.scale[j], 1.0 / (double)box.g);
+    write_cell(box, j, i, left, right, nb, out);
 }
 
-// Init-Bins (Alg. 2): nb equal bins per axis, right edges (k+1)/nb held as
+// Right edge k of Init-Bins (Alg. 2): nb equal bins, (k+1)/nb held as
 // double-double (rounded value + rounded remainder), last edge exactly 1.
-__global__ void init_grid_kernel(double* grid, double* grid_lo, int d, int nb)
+__device__ __forceinline__ DD uniform_edge(int k, int nb)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= d * nb) return;
-    const int k = i % nb;
-    if (k == nb - 1) {
-        grid[i] = 1.0;
-        grid_lo[i] = 0.0;
-        return;
-    }
+    if (k == nb - 1) return DD{1.0, 0.0};
     const double hi = __ddiv_rn((double)(k + 1), (double)nb);
     const double rem = __fma_rn(-hi, (double)nb, (double)(k + 1));  // exact
-    grid[i] = hi;
-    grid_lo[i] = __ddiv_rn(rem, (double)nb);
+    return DD{hi, __ddiv_rn(rem, (double)nb)};
+}
+
+// A problem's initial state in one launch: the uniform grid and its map cells,
+// empty histograms and iteration state (the arguments carry the tolerances,
+// so that nothing on the host has to outlive the call).
+__global__ void setup_kernel(const __grid_constant__ SetupArgs a)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) {
+        DevState* st = a.st;
+        st->it = 0;
+        st->done = st->active = st->error = st->n = st->converged = 0;
+        st->estimate = st->sigma = st->chi2_dof = 0.0;
+        st->rel_tol = a.rel_tol;
+        st->abs_tol = a.abs_tol;
+    }
+    if (i >= a.d * a.nb) return;
+    const int j = i / a.nb, k = i - j * a.nb;
+    const DD right = uniform_edge(k, a.nb), left = k ? uniform_edge(k - 1, a.nb) : DD{0.0, 0.0};
+    a.grid[i] = right.hi;
+    a.grid_lo[i] = right.lo;
+    a.hist[i] = 0.0;
+    if (i < a.hist_d * a.nb) a.hist_acc[i] = 0.0;
+    write_cell(a.box, j, i, left, right, a.nb, a.cells);
 }
 
 }  // namespace
@@ -181,10 +203,10 @@ cudaError_t launch_cells(const double* grid, const double* grid_lo, const CellBo
     return cudaGetLastError();
 }
 
-cudaError_t launch_init_grid(double* grid, double* grid_lo, int d, int nb, cudaStream_t s)
+cudaError_t launch_setup(const SetupArgs& a, cudaStream_t s)
 {
-    const int n = d * nb;
-    init_grid_kernel<<<(n + 255) / 256, 256, 0, s>>>(grid, grid_lo, d, nb);
+    const int n = a.d * a.nb;
+    setup_kernel<<<(n + 127) / 128, 128, 0, s>>>(a);
     return cudaGetLastError();
 }
 
