@@ -79,15 +79,32 @@ long long to_fixed(HD v, int f)  // v 2^f rounded, |v| 2^f < 2^63
 // width has a product shift of at least 0.  Rules per family: GAUSS sum of the
 // largest t^2 < 2^12; C0, DISCONT sum of the largest |t| < 2^9; CORNER 1 +
 // a.lo >= 1/4 and the largest sum < 2^12; PRODPEAK 1 + t^2 < 2^12 per axis;
-// OSC at most 2^6 turns per axis.
+// OSC at most 2^6 turns per axis; TABLE every axis read by one table dimension at
+// most.
 void affine_prepare(int id, const double* params, int d, const double* lo, const double* scale, long long g, int nb,
-                    FamParams* fp, CellMap* cm, double* jac0)
+                    const TableDesc* tabs, FamParams* fp, CellMap* cm, double* jac0)
 {
     fp->fix = 0;
     HD s[kDMax], a[kDMax], b[kDMax];
     HD fac{1.0, 0.0};      // f's constant factor
     double tmax[kDMax], sum = 0.0, sum2 = 0.0, most = 0.0, bmax = 0.0;
     HD start{0.0, 0.0};
+    // TABLE: the table dimension that reads each axis (at most one)
+    int knots[kDMax] = {0};
+    HD tab_lo[kDMax], tab_s[kDMax];
+    if (id == MCUBES_F_TABLE) {
+        if (!tabs) return;
+        for (int q = 0; q < fp->nf; ++q) {
+            const TableDesc& T = tabs[fp->tid[q]];
+            for (int h = 0; h < T.ndim; ++h) {
+                const int j = h ? fp->tb[q] : fp->ta[q];
+                if (knots[j]) return;  // read twice: two scales
+                knots[j] = h ? T.n1 : T.n0;
+                tab_lo[j] = HD{h ? T.lo1 : T.lo0, 0.0};
+                tab_s[j] = div(HD{(double)(knots[j] - 1), 0.0}, h ? two_sum(T.hi1, -T.lo1) : two_sum(T.hi0, -T.lo0));
+            }
+        }
+    }
     for (int j = 0; j < d; ++j) {
         double off = lo[j];  // a = s (lo - off')
         switch (id) {
@@ -97,6 +114,7 @@ void affine_prepare(int id, const double* params, int d, const double* lo, const
         case MCUBES_F_DISCONT:
         case MCUBES_F_C0: s[j] = HD{params[j], 0.0}; break;
         case MCUBES_F_PRODPEAK: s[j] = HD{std::fabs(params[j]), 0.0}; break;
+        case MCUBES_F_TABLE: s[j] = knots[j] ? tab_s[j] : div(HD{1.0, 0.0}, HD{scale[j], 0.0}); break;
         default: return;
         }
         if (!(s[j].h > 0x1p-40) || !(s[j].h < 0x1p40) || !(scale[j] > 0x1p-40) || !(scale[j] < 0x1p40)) return;
@@ -104,6 +122,7 @@ void affine_prepare(int id, const double* params, int d, const double* lo, const
         HD x0{0.0, 0.0};  // lo - o_j
         if (id == MCUBES_F_GAUSS) x0 = two_sum(off, -params[1 + j]);
         else if (id == MCUBES_F_OSC) x0 = HD{off, 0.0};
+        else if (id == MCUBES_F_TABLE) x0 = knots[j] ? two_sum(off, -tab_lo[j].h) : HD{0.0, 0.0};
         else if (id == MCUBES_F_C0 || id == MCUBES_F_PRODPEAK) x0 = two_sum(off, -params[d + j]);
         if (!(std::fabs(x0.h) < 0x1p40)) return;
         a[j] = mul(s[j], x0);
@@ -116,7 +135,7 @@ void affine_prepare(int id, const double* params, int d, const double* lo, const
         if (id == MCUBES_F_DISCONT && off != 0.0) return;  // exp(c.lo) would need an exponential of its own
         if (id == MCUBES_F_PRODPEAK) fac = mul(fac, mul(HD{params[j], 0.0}, HD{params[j], 0.0}));
     }
-    int f = 0, fq = 0;
+    int f = 0, fq = 0, fj[kDMax] = {0};
     uint64_t fu[kDMax + 1] = {0};
     switch (id) {
     case MCUBES_F_GAUSS: {
@@ -170,8 +189,19 @@ void affine_prepare(int id, const double* params, int d, const double* lo, const
         if (fq < 52) return;
         break;
     }
+    case MCUBES_F_TABLE:
+        // cell and fraction to f = 63 - (bits of the axis's range in knots): finer than u = x s - lo s in
+        // double wherever the box is not much wider than the table
+        for (int j = 0; j < d; ++j) {
+            const int tb = std::max(1, bits_above(std::max(tmax[j], b[j].h * (1.0 + 0x1p-40))));
+            fj[j] = std::min(62, 63 - tb);
+            if (knots[j] && fj[j] < 53 - bits_above((double)knots[j]) + 2) return;
+            if (fj[j] < 32) return;
+        }
+        break;
     default: return;
     }
+    if (id != MCUBES_F_TABLE) std::fill(fj, fj + d, f);
     // J f0 = prod (nb scale_j) f0 = jac0 prod W_j with W_j = (b_j / g) (unit width), as the cells hold it
     HD j0 = fac, bg[kDMax];
     for (int j = 0; j < d; ++j) {
@@ -184,8 +214,8 @@ void affine_prepare(int id, const double* params, int d, const double* lo, const
     if (lg > 31) return;
     for (int j = 0; j < d; ++j) {
         if (id == MCUBES_F_OSC) a[j] = add(a[j], HD{-std::nearbyint(a[j].h), 0.0});
-        cm->a[j] = to_fixed(a[j], f);
-        cm->b[j] = (uint64_t)to_fixed(b[j], f);
+        cm->a[j] = to_fixed(a[j], fj[j]);
+        cm->b[j] = (uint64_t)to_fixed(b[j], fj[j]);
         int e;  // b / g = m 2^(e - 63), m in [2^63, 2^64): rounded to 61 bits
         (void)std::frexp(bg[j].h, &e);
         const uint64_t v = (uint64_t)to_fixed(bg[j], 61 - e);  // 2^60..2^61
@@ -193,11 +223,14 @@ void affine_prepare(int id, const double* params, int d, const double* lo, const
         cm->bg_m[j] = v << z;
         cm->bg_e[j] = e + 2 - z;  // v 2^(e - 61) = m 2^(e - 61 - z)
     }
-    cm->fbits = f;
+    cm->on = 1;
     fp->fix = 1;
     fp->fsg = 31 - lg;
     // t = M 2^(e - 63) num 2^-33 with M num 2^fsg = H 2^64: H 2^(e - 32 - fsg), moved to f fraction bits
-    fp->ftsh = 32 + fp->fsg - f;
+    for (int j = 0; j < d; ++j) {
+        fp->ftsh[j] = 32 + fp->fsg - fj[j];
+        fp->ff[j] = fj[j];
+    }
     fp->fq = fq;
     std::copy(fu, fu + kDMax + 1, fp->fu);
     *jac0 = j0.h + j0.l;

@@ -76,7 +76,7 @@ __device__ __forceinline__ void slot_cell(const BatchDesc& D, int j, int k, DD l
 {
     const size_t i = (size_t)j * D.nb + k;
     if (D.mixed) static_cast<float2*>(D.cells)[i] = map_cell_f32(left, right, D.lo[j], D.scale[j], D.nb);
-    else if (D.cm.fbits) static_cast<double2*>(D.cells)[i] = map_cell_fix(left, right, D.cm, j);
+    else if (D.cm.on) static_cast<double2*>(D.cells)[i] = map_cell_fix(left, right, D.cm, j);
     else static_cast<double2*>(D.cells)[i] = map_cell_f64(left, right, D.lo[j], D.scale[j], inv_g);
 }
 
@@ -365,7 +365,7 @@ mcubes_status BatchEngine::admit(const mcubes_request& r, long long tag, int* sl
         D.lo[j] = r.lo[j];
         D.scale[j] = r.hi[j] - r.lo[j];
     }
-    if (!mixed_) affine_prepare(r.integrand_id, r.params, d, D.lo, D.scale, g, nb, &fp, &D.cm, &D.jac0);
+    if (!mixed_) affine_prepare(r.integrand_id, r.params, d, D.lo, D.scale, g, nb, nullptr, &fp, &D.cm, &D.jac0);
     D.fam = fp;
     const size_t grid_stride = 2 * (size_t)kDMax * nb, hist_stride = (size_t)kDMax * nb;
     D.grid = (double*)grids_.ptr + grid_stride * slot;

@@ -550,7 +550,7 @@ mcubes_status mcubes_setup(mcubes_ctx* c, int id, const double* params, int npar
     for (int j = 0; j < d; ++j) scale[j] = hi[j] - lo[j];
     CellMap cm;
     std::memset(&cm, 0, sizeof cm);
-    if (!c->mixed) affine_prepare(id, params, d, lo, scale, g, nb, &fp, &cm, &jac0);
+    if (!c->mixed) affine_prepare(id, params, d, lo, scale, g, nb, c->tabs_host.data(), &fp, &cm, &jac0);
 
     // launch shapes
     c->smem_adj = vsample_smem_bytes(c->mixed, true, d, nb, c->hist_d);

@@ -87,20 +87,21 @@ struct FamParams {
     // 0 where it does not apply
     int fix;
     int fsg;                 // left shift that brings g phi's numerator (< g 2^33) to the top of 64 bits
-    int ftsh;                // a cell width of binary exponent e moves the product right by ftsh - e
+    int ftsh[kDMax];         // axis j: a cell width of binary exponent e moves the product right by ftsh[j] - e
     int fq;                  // fraction bits of the integrand's running sum
+    int ff[kDMax];           // TABLE: fraction bits of axis j
     uint64_t fu[kDMax + 1];  // DISCONT: thresholds; [kDMax]: start of the running sum
 };
 
 // Cells of the fixed-point form: coordinate t = a + b x (x the unit-cube edge)
-// with fbits fraction bits (0: cells in the box's coordinates); a, b as such
+// with fbits[j] fraction bits (on = 0: cells in the box's coordinates); a, b as such
 // integers, b / g as bg_m 2^(bg_e - 63).  Sums wrap around 2^64 (OSC: t in
 // turns, whole ones do not matter).
 struct CellMap {
     long long a[kDMax];
     uint64_t b[kDMax], bg_m[kDMax];
     int bg_e[kDMax];
-    int fbits, pad;
+    int on, pad;
 };
 
 // Arguments of one sampling launch (Alg. 3).  Passed by value as a
@@ -228,7 +229,7 @@ struct RefineArgs {
     double* hist_acc;         // [hist_d][nb] histogram of the sampling pass; read, then cleared
     void* cells_g;            // [d][nb] map cells, rebuilt for every rebinned axis (null: none kept)
     double lo[kDMax], scale[kDMax];
-    CellMap cm;               // cm.fbits > 0: cells of the fixed-point form
+    CellMap cm;               // cm.on: cells of the fixed-point form
     double inv_g;             // 1 / g
     int mixed;
     DevState* st;
@@ -280,8 +281,9 @@ cudaError_t vsample_occupancy(int family, bool mixed, bool adjust, bool fix, int
 // the box lo + scale [0, 1]^d and fills its constants (fp's fixed-point
 // fields, the cells' coordinates, the Jacobian's constant); fp->fix = 0 and
 // *jac0 untouched where it does not.
+// tabs: the host's copies of the tables' descriptors (TABLE).
 void affine_prepare(int id, const double* params, int d, const double* lo, const double* scale, long long g, int nb,
-                    FamParams* fp, CellMap* cm, double* jac0);
+                    const TableDesc* tabs, FamParams* fp, CellMap* cm, double* jac0);
 int choose_lanes(bool mixed, long long m, long long p, long long resident);  // threads per cube
 uint64_t cube_permutation(uint64_t n);
 template <class T> void set_cube_order(T& a, uint64_t n)  // of a range of n cubes

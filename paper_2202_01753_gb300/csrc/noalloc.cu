@@ -95,7 +95,7 @@ extern "C" mcubes_status mcubes_sample_range_noalloc(
         for (int j = 0; j < d; ++j) scale[j] = hi[j] - lo[j];
         CellMap cm;
         std::memset(&cm, 0, sizeof cm);
-        if (!mixed) affine_prepare(integrand_id, params, d, lo, scale, g, nbins, &fp, &cm, &jac0);
+        if (!mixed) affine_prepare(integrand_id, params, d, lo, scale, g, nbins, nullptr, &fp, &cm, &jac0);
         const size_t smem = vsample_smem_bytes(mixed, adj, d, nbins, d);
         const size_t smem_other = vsample_smem_bytes(mixed, !adj, d, nbins, d);
         int smem_limit = 0, sms = 0, occ = 0, occ_other = 0;

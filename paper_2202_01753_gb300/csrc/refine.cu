@@ -48,7 +48,7 @@ static __device__ __forceinline__ void rebin_axis(const RefineArgs& a, int ax)
             a.grid_lo[i] = right.lo;
             if (!a.cells_g) continue;
             if (a.mixed) static_cast<float2*>(a.cells_g)[i] = map_cell_f32(left, right, a.lo[j], a.scale[j], nb);
-            else if (a.cm.fbits) static_cast<double2*>(a.cells_g)[i] = map_cell_fix(left, right, a.cm, j);
+            else if (a.cm.on) static_cast<double2*>(a.cells_g)[i] = map_cell_fix(left, right, a.cm, j);
             else static_cast<double2*>(a.cells_g)[i] = map_cell_f64(left, right, a.lo[j], a.scale[j], a.inv_g);
         }
     }
@@ -123,7 +123,7 @@ __global__ void combine_shards_kernel(const double* gathered, int nranks, int le
 __device__ __forceinline__ void write_cell(const CellBox& box, int j, int i, DD left, DD right, int nb, void* out)
 {
     if (box.mixed) static_cast<float2*>(out)[i] = map_cell_f32(left, right, box.lo[j], box.scale[j], nb);
-    else if (box.cm.fbits) static_cast<double2*>(out)[i] = map_cell_fix(left, right, box.cm, j);
+    else if (box.cm.on) static_cast<double2*>(out)[i] = map_cell_fix(left, right, box.cm, j);
     else static_cast<double2*>(out)[i] = map_cell_f64(left, right, box.lo[j], box.scale[j], 1.0 / (double)box.g);
 }
 

@@ -266,7 +266,7 @@ __device__ __forceinline__ void sample_words(const A& a, uint32_t s, const Sampl
 // The same sample in the fixed-point form (FixFamily): the cell holds t at
 // the left edge with f fraction bits and width / g as a double, of value M
 // 2^(e - 63); g phi = num 2^-33, num < g 2^33 shifted to the top of 64 bits by
-// fsg, so t = left + (M num 2^fsg) >> (64 + ftsh - e).
+// fsg, so t = left + (M num 2^fsg) >> (64 + ftsh[j] - e).
 template <int FAM, int NB4, int DC, class A>
 __device__ __forceinline__ double sample_point_fix(const A& a, const double2* cells, uint32_t s,
                                                    const SampleRng<NB4>& rng, const PhiloxCube& pc,
@@ -287,7 +287,7 @@ __device__ __forceinline__ double sample_point_fix(const A& a, const double2* ce
         const IntProd wd = int_prod_of(cell.y);
         const uint64_t num = bin_numerator(bp) << a.fam.fsg;
         const uint64_t H = __umul64hi(wd.m, num);
-        const uint32_t sh = (uint32_t)(a.fam.ftsh - wd.e);  // >= 0; beyond 63 for the narrowest bins
+        const uint32_t sh = (uint32_t)(a.fam.ftsh[j] - wd.e);  // >= 0; beyond 63 for the narrowest bins
         const int64_t t = __double_as_longlong(cell.x) + (int64_t)(sh < 64u ? H >> sh : 0ull);
         jp = int_prod_mul2(jp, wd);
         Fam::add(fs, j, t, a.fam);

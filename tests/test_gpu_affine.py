@@ -1,4 +1,4 @@
-"""The FP64 affine families, in the fixed-point form and just outside the rule
+"""The FP64 affine families and table integrands, in the fixed-point form and just outside the rule
 that selects it (csrc/affine.cu), against the oracle: boxes away from the unit
 cube, few and many bins, sub-cube counts that are and are not powers of two,
 ranges on both sides of the form's limits, negative and zero coefficients.
@@ -55,3 +55,35 @@ def test_affine_against_oracle(gpu_ctx_factory, case, lanes):
     np.testing.assert_allclose(I, o["trace_I"], rtol=0, atol=1e-12 * scale)
     np.testing.assert_allclose(V, o["trace_var"], rtol=1e-10, atol=0)
     np.testing.assert_allclose(grid, o["grid"], rtol=0, atol=1e-12)
+
+
+_rng = np.random.default_rng(17)
+TABLES = [dict(ndim=2, values=_rng.uniform(0.5, 2.0, (9, 33)), lo=(0.0, -1.0), hi=(1.0, 3.0)),
+          dict(ndim=1, values=_rng.uniform(0.5, 2.0, 1000), lo=0.25, hi=0.75),
+          dict(ndim=1, values=np.array([1.0, 3.0]), lo=-2.0, hi=5.0)]
+TABLE_CASES = [
+    # factors (table, axis, second axis), lo, hi: boxes inside, beside and across the knot ranges
+    ("one_factor_each", [(0, 1, 0), (1, 2, -1), (2, 3, -1)], [-1.5, -0.5, 0.0, -3.0], [3.5, 1.5, 1.0, 6.0]),
+    ("outside", [(1, 0, -1), (2, 1, -1)], [0.8, 7.0], [0.9, 8.0]),
+    ("flat_axis", [(2, 1, -1)], [0.0, 0.0, 0.0], [1.0, 1.0, 1.0]),
+    ("read_twice", [(0, 0, 1), (1, 0, -1)], [0.0, 0.0], [1.0, 1.0]),
+    ("wide_box", [(1, 0, -1)], [-1e6, 0.0], [1e6, 1.0]),
+    ("six_factors", [(2, j, -1) for j in range(6)], [0.0] * 6, [1.0] * 6),
+]
+
+
+@pytest.mark.parametrize("case", TABLE_CASES, ids=[c[0] for c in TABLE_CASES])
+def test_tables_against_oracle(gpu_ctx_factory, case):
+    _, factors, lo, hi = case
+    params = np.array([-0.5, len(factors)] + [v for f in factors for v in f], dtype=np.float64)
+    lo, hi = np.array(lo), np.array(hi)
+    oracle.set_tables(TABLES)
+    o = oracle.integrate(W.F_TABLE, params, lo, hi, 30_000, 4, nb=200, seed=22)
+    ctx = gpu_ctx_factory(nbins=200, seed=22)
+    ctx.set_tables(TABLES)
+    ctx.integrate(W.F_TABLE, params, lo, hi, 30_000, 4)
+    I, V = ctx.trace()
+    ctx.close()
+    np.testing.assert_allclose(I, o["trace_I"], rtol=0, atol=1e-12 * np.max(np.abs(o["trace_I"])))
+    # a constant region's variance is rounding: beside the estimate's own last places
+    np.testing.assert_allclose(V, o["trace_var"], rtol=1e-10, atol=1e-28 * np.max(o["trace_I"] ** 2))
