@@ -134,8 +134,7 @@ __device__ void refine_one(const BatchRefineArgs& a, uint32_t j, RebinShared& sh
             // the histogram: the sum of the integral's segments in their order
             double acc = 0.0;
             if (a.hist_is_float) {
-                const float* ph = reinterpret_cast<const float*>(parts) + k;
-                for (int b = 0; b < nparts; ++b) acc += (double)ph[b * stride];
+                acc = fx::fx_sum_floats(reinterpret_cast<const uint32_t*>(parts) + k, stride, nparts);
             } else {
                 const double* ph = reinterpret_cast<const double*>(parts) + k;
                 for (int b = 0; b < nparts; ++b) acc += ph[b * stride];
@@ -438,14 +437,17 @@ void BatchEngine::live_slots(std::vector<int>* live, ClassMask* class_mask) cons
 // per block, the serving mix without retries at 2000 requests/s p50 2.6 ms and
 // p99 3.9 ms against 15.2 and 21.0; 8192: 3.1 and 4.1 ms, 32768: 7.1 and 8.5).
 constexpr double kMinBlockSamples = 2048.0;
-// A step's chunks, all classes together, fill about kChunkWaves waves of the
-// GPU's resident blocks (three 256-thread blocks per SM); beyond that chunks
-// grow, up to kMaxChunkSamples, so that a block's fixed work (~5 us: staging a
-// segment, writing its histogram) stays small beside its samples.  256
-// requests of 1e5 calls: 20.8 -> 15.6 ms against chunks of 2048 samples
-// (3 waves 16.0, 12 waves 18.1 ms); 1024 integrals of 1e4-1e7 calls, whose
-// chunks would be 2.6e5 samples at 6 waves: 106.6 ms, 105.2 at 12 waves
-// (a finer tail), hence the upper limit.
+// In double precision a step's chunks, all classes together, fill about
+// kChunkWaves waves of the GPU's resident blocks (three 256-thread blocks per
+// SM); beyond that chunks grow, up to kMaxChunkSamples, so that a block's fixed
+// work (~5 us: staging a segment, writing its histogram) and the merge of its
+// histogram stay small beside its samples: 256 requests of 1e5 calls 37.8
+// -> 32.2 ms against chunks of 2048 samples (12 waves 36.4), 256 integrals of
+// 1e4-1e6 calls 11.4 -> 9.8 ms.  In single precision a chunk's histogram is
+// summed in floats and its length decides their rounding: there the chunks stay
+// as short as the occupancy lets them (the longer ones would take 256 requests
+// of 1e5 calls from 17.9 to 13.4 ms, with 2.5-4 times the run-to-run spread
+// between the chi-squares of the two).
 constexpr double kChunkWaves = 6.0;
 constexpr double kMaxChunkSamples = 32768.0;
 
@@ -470,7 +472,8 @@ void BatchEngine::partition(const std::vector<int>& live, int* nseg_out)
     double all = 0.0;
     for (int s : live) all += slots_[s].work;
     const double chunk_min =
-        std::min(std::max(kMinBlockSamples, all / (kChunkWaves * 3.0 * num_sms_)), kMaxChunkSamples);
+        mixed_ ? kMinBlockSamples
+               : std::min(std::max(kMinBlockSamples, all / (kChunkWaves * 3.0 * num_sms_)), kMaxChunkSamples);
     while (j < live.size()) {
         const int cls = batch_class(hdesc_[live[j]].family, (int)hdesc_[live[j]].d);
         size_t j1 = j;

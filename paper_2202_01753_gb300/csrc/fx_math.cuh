@@ -314,6 +314,54 @@ __device__ __forceinline__ float rcp_seed(float x)
 #endif
 }
 
+// The sum of n non-negative floats at p[0], p[stride], ... (as bits), to a
+// double: 24-bit mantissas added as 128-bit integers, placed so that n of them
+// at the largest exponent so far cannot overflow; nothing above 2^-100 of the
+// largest is lost, and the sum is rounded at the end.  In double precision each
+// addend is a conversion and an addition at 2 lanes per clock and SM: merging
+// the partial histograms of 256 integrals of 1e5 calls, 49 parts each, took
+// 110 us of an iteration there (the whole call 19.1 -> 17.8 ms, 64 integrals of
+// 1e4-1e6 calls 3.70 -> 3.02 ms).  Infinities and NaN go that way still.
+__device__ __forceinline__ double fx_sum_floats(const uint32_t* p, size_t stride, int n)
+{
+    using u128 = unsigned __int128;
+    constexpr int kAhead = 8;  // loads in flight (16: the same)
+    const int top = 40 - (n > 1 ? 64 - __clzll((long long)n - 1) : 0);
+    u128 acc = 0;
+    uint32_t E = 1;  // acc counts units of 2^(E - 150 - top - 64)
+    bool plain = top < 8;
+    for (int b = 0; b < n && !plain; b += kAhead) {
+        uint32_t u[kAhead], mx = 0;
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) u[i] = b + i < n ? p[(size_t)(b + i) * stride] : 0u;
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) mx = u[i] > mx ? u[i] : mx;
+        plain = mx >= 0x7F800000u;
+        const uint32_t e = mx >> 23;
+        if (e > E) {
+            acc = e - E < 128u ? acc >> (e - E) : (u128)0;
+            E = e;
+        }
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
+            const uint32_t ei = u[i] >> 23 ? u[i] >> 23 : 1u, sh = E - ei;
+            const uint64_t m = (uint64_t)(u[i] - ((ei - 1u) << 23)) << top;  // the implicit bit with it
+            acc += sh < 128u ? (u128)m << 64 >> sh : (u128)0;  // (after an infinity or NaN: not used)
+        }
+    }
+    if (plain) {
+        double s = 0.0;
+        for (int b = 0; b < n; ++b) {
+            float f;
+            memcpy(&f, &p[(size_t)b * stride], 4);
+            s += (double)f;
+        }
+        return s;
+    }
+    const double unit = __longlong_as_double((long long)((int)E - 150 - top + 1023) << 52);  // of the upper word
+    return (double)(uint64_t)(acc >> 64) * unit + (double)(uint64_t)acc * (unit * 5.421010862427522e-20);  // 2^-64
+}
+
 // 2^64 / x for x = m 2^-63 in [1, 2), by two Newton-Raphson steps y (2 - x y)
 // in fixed point from a single-precision seed kept below 1/x, so that every
 // residual is non-negative: relative error below 2^-60.  Returns a value in
