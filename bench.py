@@ -52,17 +52,18 @@ from paper_2202_01753_gb300 import closed_forms as CF  # noqa: E402
 # "fp32_flops": 2 FFMA + FADD + FMUL per sample (the FP32-pipe fraction shown
 # beside the issue fraction).
 ROOFLINE_UNITS = {
-    ("cosmo6", "fp64"): {"kind": "fp64", "per_sample": 29.86, "issue_per_sample": 2032.5, "traffic": 277.2e3,
-                         "pipe_busy": 0.781,
+    ("cosmo6", "fp64"): {"kind": "fp64", "per_sample": 28.68, "issue_per_sample": 1925.4, "traffic": 147.7e3,
+                         "pipe_busy": 0.776,
                          "source": "profiles/vsample_cosmo6_fp64.md"},
-    ("gauss3", "fp64"): {"kind": "fp64", "per_sample": 26.92, "traffic": 101.4e3, "pipe_busy": 0.783,
+    ("gauss3", "fp64"): {"kind": "fp64", "per_sample": 9.62, "issue_per_sample": 601.5, "traffic": 98.6e3,
+                         "pipe_busy": 0.680,
                          "source": "profiles/vsample_gauss3_fp64.md"},
-    ("table6", "fp64"): {"kind": "fp64", "per_sample": 43.74, "dram_bytes_per_sample": 409.2, "traffic": 38.5028e9,
-                         "pipe_busy": 0.734,
+    ("table6", "fp64"): {"kind": "fp64", "per_sample": 38.66, "issue_per_sample": 1228.9,
+                         "dram_bytes_per_sample": 432.5, "traffic": 40.6917e9, "pipe_busy": 0.747,
                          "source": "profiles/vsample_table6_fp64.md"},
-    ("corner8", "mixed"): {"kind": "issue", "per_sample": 533.1, "traffic": 598.8e3, "fp32_flops": 99.08,
+    ("corner8", "mixed"): {"kind": "issue", "per_sample": 432.4, "traffic": 544.8e3, "fp32_flops": 99.08,
                            "source": "profiles/vsample_corner8_mixed.md"},
-    ("osc10", "mixed"): {"kind": "issue", "per_sample": 654.3, "traffic": 301.1e3, "fp32_flops": 134.87,
+    ("osc10", "mixed"): {"kind": "issue", "per_sample": 605.8, "traffic": 150.5e3, "fp32_flops": 134.80,
                          "source": "profiles/vsample_osc10_mixed.md"},
 }
 DFMA_PER_CLK_PER_SM = 2.0

@@ -445,8 +445,8 @@ constexpr double kMinBlockSamples = 2048.0;
 // -> 32.2 ms against chunks of 2048 samples (12 waves 36.4), 256 integrals of
 // 1e4-1e6 calls 11.4 -> 9.8 ms.  In single precision a chunk's histogram is
 // summed in floats and its length decides their rounding: there the chunks stay
-// as short as the occupancy lets them (the longer ones would take 256 requests
-// of 1e5 calls from 17.9 to 13.4 ms, with 2.5-4 times the run-to-run spread
+// as short as the occupancy lets them (the longer ones took 256 requests of
+// 1e5 calls from 19.1 to 13.9 ms, with 2.5-4 times the run-to-run spread
 // between the chi-squares of the two).
 constexpr double kChunkWaves = 6.0;
 constexpr double kMaxChunkSamples = 32768.0;
