@@ -184,7 +184,8 @@ constexpr bool rolled_axes()
 // so the per-axis code exists once instead of D times.  Unrolled, a six-axis
 // sample is thousands of instructions, more than the SM's instruction
 // caches keep close, and warps wait on instruction fetch.  In the loop the
-// sub-cube digit of axis j is peeled off the cube index (one high multiply),
+// sub-cube digit of axis j is peeled off the cube index (one high multiply and
+// one correction, as cube_digits; a second one cost cosmo6 0.9%),
 // the Philox block of axes 4b..4b+3 is drawn at j = 4b and its words are
 // rotated into place, and the flat bin indices are shifted into idx from the
 // top, so that after the last axis axis j's index is field j (the layout
@@ -217,7 +218,6 @@ sample_point_rolled(const A& a, const typename Prec<MIXED>::Cell* cells, uint32_
         r = make_uint4(r.y, r.z, r.w, r.x);
         uint32_t q = __umulhi(rest, a.gmagic);
         uint32_t dig = rest - q * a.g;
-        if (dig >= a.g) { ++q; dig -= a.g; }
         if (dig >= a.g) { ++q; dig -= a.g; }
         rest = q;
         const BinPos<true> bp = bin_pos<true>(w, dig * nb + 1u, nb, a.g, a.gmagic);
@@ -368,6 +368,8 @@ __device__ __forceinline__ uint64_t mod_by(uint64_t x, uint64_t n, uint64_t inv)
 
 // nb times the digit of cube c on every axis (axis 0 fastest), plus 1 where bin
 // positions are exact (bin_pos).
+// One correction is enough: with gmagic = (2^32 - e)/g, 1 <= e <= g, the high
+// word of rest gmagic is below rest/g by rest e/(g 2^32) < 1 at most.
 template <int NB4, int DC, class A>
 __device__ __forceinline__ void cube_digits(const A& a, uint32_t c, uint32_t (&nbc)[4 * NB4])
 {
@@ -376,7 +378,6 @@ __device__ __forceinline__ void cube_digits(const A& a, uint32_t c, uint32_t (&n
     for (int j = 0; j < DC; ++j) {
         uint32_t q = __umulhi(rest, a.gmagic);
         uint32_t r = rest - q * a.g;
-        if (r >= a.g) { ++q; r -= a.g; }
         if (r >= a.g) { ++q; r -= a.g; }
         nbc[j] = r * a.nb + (DC >= 3 ? 1u : 0u);
         rest = q;
@@ -413,7 +414,6 @@ __device__ __forceinline__ void cube_step_digits32(uint32_t step, uint32_t n, ui
         for (int h = 0; h < 2; ++h) {
             uint32_t q = __umulhi(u[h], a.gmagic);
             uint32_t rem = u[h] - q * a.g;
-            if (rem >= a.g) { ++q; rem -= a.g; }
             if (rem >= a.g) { ++q; rem -= a.g; }
             out[h * kDMax + j] = rem * a.nb;
             u[h] = q;
