@@ -52,8 +52,8 @@ from paper_2202_01753_gb300 import closed_forms as CF  # noqa: E402
 # "fp32_flops": 2 FFMA + FADD + FMUL per sample (the FP32-pipe fraction shown
 # beside the issue fraction).
 ROOFLINE_UNITS = {
-    ("cosmo6", "fp64"): {"kind": "fp64", "per_sample": 28.68, "issue_per_sample": 1925.4, "traffic": 147.7e3,
-                         "pipe_busy": 0.776,
+    ("cosmo6", "fp64"): {"kind": "fp64", "per_sample": 28.68, "issue_per_sample": 1895.5, "traffic": 147.7e3,
+                         "pipe_busy": 0.782,
                          "source": "profiles/vsample_cosmo6_fp64.md"},
     ("gauss3", "fp64"): {"kind": "fp64", "per_sample": 9.62, "issue_per_sample": 601.5, "traffic": 98.6e3,
                          "pipe_busy": 0.680,
