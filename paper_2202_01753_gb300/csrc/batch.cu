@@ -101,22 +101,16 @@ __device__ void refine_one(const BatchRefineArgs& a, uint32_t j, RebinShared& sh
     const uint32_t slot = a.live[j];
     const BatchDesc& D = a.desc[slot];
     const uint32_t s0 = a.live_seg[j], s1 = a.live_seg[j + 1];
+    // finished in an earlier iteration of this step: its sampling was skipped.
+    // The sampling launch's own record decides, not the state, which this
+    // launch's finalising block (and a rebinning block that meets a non-finite
+    // sum) writes while the integral's other blocks start.
+    if (!a.segs[s0].ran) return;
     const bool adjust = a.segs[s0].adjust != 0;
     const int d = (int)D.d, nb = (int)D.nb;
     const int nrebin = adjust ? d : 0;
     if ((int)blockIdx.x > nrebin) return;
     BatchState* st = a.st + slot;
-    // finished in an earlier iteration of this step (its sampling was skipped).
-    // The finalising block of this launch may set these while a rebinning
-    // block reads them: that block then skips a rebin no iteration will use.
-    // One thread reads, so that the whole block takes the same branch.
-    __shared__ int skip;
-    if (threadIdx.x == 0)
-        skip = *(volatile const int*)&st->done || (int)*(volatile const uint32_t*)&st->it >= D.itmax;
-    __syncthreads();
-    const bool finished = skip != 0;
-    __syncthreads();  // skip is rewritten for the next integral
-    if (finished) return;
     if ((int)blockIdx.x == nrebin) {
         const IterRecord r{&st->it, &st->done, &st->error, &st->n, &st->converged, &st->estimate, &st->sigma,
                            &st->chi2_dof, D.hist_I, D.hist_V, D.itmax, D.rel_tol, D.abs_tol};
@@ -511,6 +505,7 @@ void BatchEngine::partition(const std::vector<int>& live, int* nseg_out)
                     BatchSeg& g = h_segs_[nseg++];
                     g.slot = (uint32_t)s;
                     g.adjust = adjust ? 1u : 0u;
+                    g.ran = 0u;
                     g.c0 = c;
                     g.c1 = cend;
                     set_cube_order(g, cend - c);

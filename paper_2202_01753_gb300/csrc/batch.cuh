@@ -64,12 +64,16 @@ vsample_batch_kernel(const __grid_constant__ BatchArgs a)
         stage_cells<MIXED>(cells, static_cast<const unsigned char*>(a.cells) + a.cell_stride * seg.slot, D, a.nb);
         __syncthreads();
         // an integral that finished in an earlier iteration of this step (a
-        // step may run several) is skipped; only the refinement changes the state
-        if (now.y || now.x >= sd.itmax) continue;
-        // this iteration adjusts while it < ita (a step's iterations may cross
-        // ita); the refinement reads the flag back
-        const bool adjust = seg.adjust && now.x < sd.ita;
-        if (threadIdx.x == 0) a.segs[si].adjust = adjust ? 1u : 0u;
+        // step may run several) is skipped; only the refinement changes the state.
+        // This iteration adjusts while it < ita (a step's iterations may cross
+        // ita).  The refinement reads both flags back.
+        const bool run = !now.y && now.x < sd.itmax;
+        const bool adjust = run && seg.adjust && now.x < sd.ita;
+        if (threadIdx.x == 0) {
+            a.segs[si].ran = run ? 1u : 0u;
+            a.segs[si].adjust = adjust ? 1u : 0u;
+        }
+        if (!run) continue;
         constexpr uint32_t d = D;
         const uint32_t nb = a.nb;
         FamParams uf;  // single precision: the integrand's constants (those it reads)

@@ -184,12 +184,13 @@ struct BatchSeg {
     uint64_t c0, c1;
     uint64_t perm_k, perm_inv;  // cube order within the segment (see sample_cubes)
     uint64_t hist_off;          // element offset of the segment's partial histogram
+    uint32_t ran, pad;          // device: sampled in this iteration (0: the integral had finished)
 };
 
 struct BatchArgs {
     const BatchDesc* desc;
     const BatchState* st;
-    BatchSeg* segs;             // the sampling launch sets each segment's adjust for this iteration
+    BatchSeg* segs;             // the sampling launch sets each segment's ran and adjust for this iteration
     const uint32_t* blk_seg;    // block b samples segments [blk_seg[b], blk_seg[b+1]) (this class's table)
     double* seg_part;           // [segment][3] partial sums
     void* seg_hist;             // partial histograms (float in mixed, double in fp64)
