@@ -294,8 +294,11 @@ cudaError_t BatchEngine::reserve(int capacity, int itcap)
 
 int BatchEngine::choose_lanes(long long p) const
 {
-    if (opts_.lanes_per_cube > 0) return (int)std::min<long long>(opts_.lanes_per_cube, std::max<long long>(p, 1));
     int L = 1;
+    if (opts_.lanes_per_cube > 0) {  // at most p, and a power of two as the sampling loop's masks and shuffles need
+        while (2 * L <= opts_.lanes_per_cube && 2 * L <= p) L *= 2;
+        return L;
+    }
     while (L < 32 && 2 * L <= p && p / L > lanes_cap_) L *= 2;
     return L;
 }
