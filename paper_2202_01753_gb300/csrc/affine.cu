@@ -77,7 +77,10 @@ long long to_fixed(HD v, int f)  // v 2^f rounded, |v| 2^f < 2^63
 // form's; negative coefficients, flat axes, and wide or far boxes keep that
 // form.  An axis's whole range of t is below 2^(63 - f), so that a cell of any
 // width has a product shift of at least 0.  Rules per family: GAUSS sum of the
-// largest t^2 < 2^12; C0, DISCONT sum of the largest |t| < 2^9; CORNER 1 +
+// largest t^2 < 2^12; C0, DISCONT sum of the largest |t| < 2^9, and a cut inside
+// the box at t >= 2^55 units of 2^-f (the threshold and a sample's t are within
+// three units: less than the last place of x, where the double-precision form
+// puts it); CORNER 1 +
 // a.lo >= 1/4 and the largest sum < 2^12; PRODPEAK 1 + t^2 < 2^12 per axis;
 // OSC at most 2^6 turns per axis; TABLE every axis read by one table dimension at
 // most.
@@ -157,9 +160,11 @@ void affine_prepare(int id, const double* params, int d, const double* lo, const
         if (id == MCUBES_F_DISCONT) {
             if (!(sum < 700.0)) return;  // exp could overflow: the double-precision form reports it
             for (int j = 0; j < d; ++j) {  // x < w_j: t < c_j w_j (lo = 0)
-                const HD t = mul(s[j], HD{params[d + j], 0.0});
-                if (!(t.h > 0.0)) fu[j] = 0;                       // always out
-                else if (t.h > tmax[j]) fu[j] = ~0ull;       // always in
+                const double w = params[d + j];
+                const HD t = mul(s[j], HD{w, 0.0});
+                if (!(w > 0.0)) fu[j] = 0;                   // always out
+                else if (w >= scale[j]) fu[j] = ~0ull;       // always in
+                else if (std::ldexp(t.h, f) < 0x1p55) return;  // an axis flat beside the others: a cut as coarse as f
                 else fu[j] = (uint64_t)to_fixed(t, f);
             }
         }
