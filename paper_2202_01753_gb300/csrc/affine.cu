@@ -71,19 +71,26 @@ long long to_fixed(HD v, int f)  // v 2^f rounded, |v| 2^f < 2^63
 }  // namespace
 
 // The fixed-point form applies where every axis really is scaled (positive
-// coefficients of a sane size) and the running quantity keeps at least 52
-// fraction bits (2^12 range), i.e. at least a double's absolute precision
-// next to 1, so that no result is less exact than the double-precision
-// form's; negative coefficients, flat axes, and wide or far boxes keep that
-// form.  An axis's whole range of t is below 2^(63 - f), so that a cell of any
-// width has a product shift of at least 0.  Rules per family: GAUSS sum of the
-// largest t^2 < 2^12; C0, DISCONT sum of the largest |t| < 2^9, and a cut inside
-// the box at t >= 2^55 units of 2^-f (the threshold and a sample's t are within
-// three units: less than the last place of x, where the double-precision form
-// puts it); CORNER 1 +
-// a.lo >= 1/4 and the largest sum < 2^12; PRODPEAK 1 + t^2 < 2^12 per axis;
-// OSC at most 2^6 turns per axis; TABLE every axis read by one table dimension at
-// most.
+// coefficients of a sane size) and the running quantity's unit is small enough
+// for results no less exact than the double-precision form's: negative
+// coefficients, flat axes, and wide or far boxes keep that form.  A sample's t
+// is its cell's left edge rounded to nearest plus a product cut downwards; the
+// running sums start with the half units that their terms lose on average, so
+// that what is left of an estimate's error is below a double's last place
+// (tests/test_affine_host.py; without them, 12 axes of |t| or of a corner
+// family's slopes 300 put the mean off by 5-9e-16 relative).  An axis's whole
+// range of t is below 2^(63 - f), so that a cell of any width has a product
+// shift of at least 0.  Rules per family:
+//   GAUSS    sum of the largest t^2 < 2^12 (unit of the exponent 2^-52)
+//   C0       sum of the largest |t| < 2^9 (2^-54)
+//   DISCONT  the same, and a cut inside the box at t >= 2^55 units (the threshold
+//            and a sample's t are within three: less than the last place of
+//            x, where the double-precision form puts it)
+//   CORNER   largest sum < 2^12, and 1 + a.lo >= 2^56 units: the power d + 1
+//            multiplies the sum's relative error (from 1, sums below 128)
+//   PRODPEAK 1 + t^2 < 2^12 per axis
+//   OSC      at most 2^6 turns per axis
+//   TABLE    every axis read by one table dimension at most
 void affine_prepare(int id, const double* params, int d, const double* lo, const double* scale, long long g, int nb,
                     const TableDesc* tabs, FamParams* fp, CellMap* cm, double* jac0)
 {
@@ -157,6 +164,7 @@ void affine_prepare(int id, const double* params, int d, const double* lo, const
         const int qb = std::max(1, bits_above(std::max(sum, bmax)));
         if (qb > 9) return;
         f = fq = 63 - qb;
+        fu[kDMax] = (uint64_t)d / 2;  // the d terms are cut, by half a unit each on average
         if (id == MCUBES_F_DISCONT) {
             if (!(sum < 700.0)) return;  // exp could overflow: the double-precision form reports it
             for (int j = 0; j < d; ++j) {  // x < w_j: t < c_j w_j (lo = 0)
@@ -173,9 +181,9 @@ void affine_prepare(int id, const double* params, int d, const double* lo, const
     case MCUBES_F_CORNER: {
         start = add(start, HD{1.0, 0.0});
         const int qb = std::max(1, bits_above((start.h + sum) * (1.0 + 0x1p-40)));
-        if (!(start.h >= 0.25) || qb > 12) return;
         f = fq = 63 - qb;
-        fu[kDMax] = (uint64_t)to_fixed(start, f);
+        if (qb > 12 || !(std::ldexp(start.h, f) >= 0x1p56)) return;
+        fu[kDMax] = (uint64_t)to_fixed(add(start, HD{std::ldexp(0.5 * d, -f), 0.0}), f);  // the terms are cut as C0's
         break;
     }
     case MCUBES_F_OSC: {

@@ -302,8 +302,8 @@ __device__ __forceinline__ double2 map_cell_f64(DD left, DD right, double lo, do
     return make_double2(lo + scale * left.hi, scale * wd * inv_g);
 }
 
-// Map cell of the fixed-point form: (t at the left edge as an integer with
-// a few tens of fraction bits, t width / g as a double), in integers but for none.
+// Map cell of the fixed-point form, in integers: (t at the left edge as an
+// integer with 51 to 62 fraction bits, rounded to nearest, and t width / g as a double).
 __device__ __forceinline__ double2 map_cell_fix(DD left, DD right, const CellMap& m, int j)
 {
     const int E = exponent_of(right.hi);
@@ -315,9 +315,11 @@ __device__ __forceinline__ double2 map_cell_fix(DD left, DD right, const CellMap
         width = int_prod_value(int_prod_mul2(IntProd{(uint64_t)((w << z) >> 64), E + 1 - z},
                                              IntProd{m.bg_m[j], m.bg_e[j]}));
     }
-    const int sh = 62 - E;  // the left edge (< 1) as Q64
-    const uint64_t l64 = sh < 128 ? (uint64_t)(lu >> sh) : 0ull;
-    return make_double2(__longlong_as_double(m.a[j] + (long long)__umul64hi(m.b[j], l64)), width);
+    const int sh = 62 - E;  // the left edge (< 1) as Q64, rounded where that stays below 1
+    uint64_t l64 = sh < 128 ? (uint64_t)(lu >> sh) : 0ull;
+    if (sh <= 128 && l64 != ~0ull) l64 += (uint64_t)(lu >> (sh - 1)) & 1ull;
+    const uint64_t t = __umul64hi(m.b[j], l64) + ((m.b[j] * l64) >> 63);
+    return make_double2(__longlong_as_double(m.a[j] + (long long)t), width);
 }
 
 __device__ __forceinline__ float2 map_cell_f32(DD left, DD right, double lo, double scale, uint32_t nb)
@@ -757,8 +759,9 @@ template <> struct FixFamily<MCUBES_F_GAUSS> {
 template <> struct FixFamily<MCUBES_F_C0> {
     static constexpr bool kHas = true;
     using S = FixSum;
-    __device__ static void begin(S& s, const FamParams&) { s.q = 0; }
-    __device__ static void add(S& s, int, int64_t t, const FamParams&) { s.q += abs_u64(t); }
+    __device__ static void begin(S& s, const FamParams& f) { s.q = f.fu[kDMax]; }
+    // |t|, or one less on the negative side: t is cut downwards, so both sides are short by half a unit on average
+    __device__ static void add(S& s, int, int64_t t, const FamParams&) { s.q += (uint64_t)(t ^ (t >> 63)); }
     template <int D> __device__ static double end(const S& s, const FamParams& f, const IntProd& jp)
     {
         return fx::fx_exp_fixed<true>(s.q, f.fq, jp.m, jp.e);
@@ -771,9 +774,9 @@ template <> struct FixFamily<MCUBES_F_DISCONT> {
         uint64_t q;
         bool out;
     };
-    __device__ static void begin(S& s, const FamParams&)
+    __device__ static void begin(S& s, const FamParams& f)
     {
-        s.q = 0;
+        s.q = f.fu[kDMax];
         s.out = false;
     }
     __device__ static void add(S& s, int j, int64_t t, const FamParams& f)

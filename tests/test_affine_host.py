@@ -51,3 +51,21 @@ def test_discont_ordinary_cuts_keep_the_fixed_form(affine):
     # cuts at or beyond the box's sides need no resolution
     for cut in (-0.5, 0.0, 1.0, 1.5):
         assert affine("fix", W.F_DISCONT, [1e-10, 60.0, cut, 0.5], [0.0] * 2, [1.0] * 2)[0] == 1
+
+
+C0, CO, DI = W.F_C0, W.F_CORNER, W.F_DISCONT
+MEANS = [(CO, [300.0] * 12), (CO, [600.0] * 6), (CO, [1300.0] * 3), (CO, [10.0] * 12), (CO, [11.0] * 11), (CO, [1.0] * 6),
+         (CO, [126.0]), (C0, [40.0] * 12 + [0.0] * 12), (C0, [40.0] * 12 + [1.0] * 12), (C0, [40.0] * 11 + [0.0] * 11),
+         (C0, [40.0] * 12 + [0.5] * 12), (C0, [170.0] * 3 + [0.0] * 3), (C0, [500.0, 0.0]),
+         (DI, [40.0] * 12 + [2.0] * 12), (DI, [40.0] * 11 + [2.0] * 11), (DI, [170.0] * 3 + [0.9] * 3)]
+
+
+@pytest.mark.parametrize("power", [1.0, 3.0])
+@pytest.mark.parametrize("case", range(len(MEANS)))
+def test_mean_error(affine, case, power):
+    """The mean of F over 60,000 samples, even and corner-ward edges, at the ends of the form's ranges: relative
+    error below one last place of a double, or the double-precision form's where that is larger."""
+    fid, params = MEANS[case]
+    d = len(params) if fid == CO else len(params) // 2
+    _, err, err_double = affine("mean", fid, params, [0.0] * d, [1.0] * d, n=60000, power=power)
+    assert abs(err) <= max(2.0 ** -52, abs(err_double))
