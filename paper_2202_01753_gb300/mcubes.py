@@ -431,8 +431,8 @@ def _requests(requests):
     addr = flat.ctypes.data + 8 * (np.cumsum(sizes) - sizes)
     rec = np.frombuffer(arr, dtype=_REQUEST)
     rec["params"], rec["lo"], rec["hi"] = addr[0::3], addr[1::3], addr[2::3]
-    rec["nparams"] = [len(p) for p in parts[0::3]]
-    rec["d"] = [len(p) for p in parts[1::3]]
+    counts = [len(p) if p.ndim else 1 for p in parts]  # a scalar is one element
+    rec["nparams"], rec["d"] = counts[0::3], counts[1::3]
     rec["integrand_id"] = [_wrap(r["fid"], 32) for r in reqs]
     rec["itmax"] = [_wrap(r["itmax"], 32) for r in reqs]
     rec["ncall"] = [_wrap(r["ncall"], 64) for r in reqs]
