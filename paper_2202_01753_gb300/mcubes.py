@@ -431,7 +431,9 @@ def _requests(requests):
     addr = flat.ctypes.data + 8 * (np.cumsum(sizes) - sizes)
     rec = np.frombuffer(arr, dtype=_REQUEST)
     rec["params"], rec["lo"], rec["hi"] = addr[0::3], addr[1::3], addr[2::3]
-    counts = [len(p) if p.ndim else 1 for p in parts]  # a scalar is one element
+    counts = np.array([len(p) if p.ndim else 1 for p in parts], dtype=np.uintp)  # a scalar is one element
+    if (sizes < counts).any() or (sizes[2::3] < counts[1::3]).any():
+        raise ValueError("a request's hi has fewer values than its lo, or an array has fewer values than rows")
     rec["nparams"], rec["d"] = counts[0::3], counts[1::3]
     rec["integrand_id"] = [_wrap(r["fid"], 32) for r in reqs]
     rec["itmax"] = [_wrap(r["itmax"], 32) for r in reqs]

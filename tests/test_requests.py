@@ -19,3 +19,14 @@ def test_scalars_are_one_element():
     assert [_values(a) for a in arr] == [(0, [2.5], [-1.0], [3.0], 100, 2, 0.0, 0.0, 0),
                                          (1, [1.0, 0.5, 0.25], [0.0], [1.0], 100000, 3, 1e-3, 2.0, 9),
                                          (0, [7.0], [0.0], [1.0], 100, 2, 0.0, 0.0, 0)]
+
+
+def test_short_arrays_are_refused():
+    """The library reads as many hi as lo values: the ones after a shorter hi are another request's."""
+    ok = dict(fid=0, params=[1.0], lo=[0.0, 0.0], hi=[1.0, 1.0], ncall=100, itmax=2)
+    for bad in (dict(hi=[1.0]), dict(hi=1.0), dict(hi=[]), dict(lo=np.zeros((2, 0))), dict(params=np.zeros((3, 0)))):
+        for reqs in ([{**ok, **bad}], [{**ok, **bad}, ok], [ok, {**ok, **bad}]):
+            with pytest.raises(ValueError):
+                mcubes._requests(reqs)
+    arr, _ = mcubes._requests([{**ok, "hi": [1.0, 2.0, 3.0]}])  # more than it reads
+    assert _values(arr[0])[2:4] == ([0.0, 0.0], [1.0, 2.0])
