@@ -8,6 +8,7 @@ there is no other implementation to fall back to.
 from __future__ import annotations
 
 import ctypes
+import operator
 import os
 import threading
 
@@ -435,7 +436,7 @@ def _requests(requests):
     if (sizes < counts).any() or (sizes[2::3] < counts[1::3]).any():
         raise ValueError("a request's hi has fewer values than its lo, or an array has fewer values than rows")
     rec["nparams"], rec["d"] = counts[0::3], counts[1::3]
-    rec["integrand_id"] = [_wrap(r["fid"], 32) for r in reqs]
+    rec["integrand_id"] = [_wrap(operator.index(r["fid"]), 32) for r in reqs]  # no float or text
     rec["itmax"] = [_wrap(r["itmax"], 32) for r in reqs]
     rec["ncall"] = [_wrap(r["ncall"], 64) for r in reqs]
     rec["rel_tol"] = [float(r.get("rel_tol", 0.0)) for r in reqs]

@@ -30,3 +30,12 @@ def test_short_arrays_are_refused():
                 mcubes._requests(reqs)
     arr, _ = mcubes._requests([{**ok, "hi": [1.0, 2.0, 3.0]}])  # more than it reads
     assert _values(arr[0])[2:4] == ([0.0, 0.0], [1.0, 2.0])
+
+
+def test_fid_is_an_integer():
+    ok = dict(fid=0, params=[1.0], lo=[0.0], hi=[1.0], ncall=100, itmax=2)
+    for fid in (1.0, 1.9, np.float64(2.0), "1", None):
+        with pytest.raises(TypeError):
+            mcubes._requests([{**ok, "fid": fid}])
+    for fid in (1, np.int32(1), np.int64(1), True):
+        assert mcubes._requests([{**ok, "fid": fid}])[0][0].integrand_id == 1
