@@ -41,7 +41,7 @@ vsample_batch_kernel(const __grid_constant__ BatchArgs a)
     using HT = typename Prec<MIXED>::H;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double red[3][kVsThreads / 32];
-    __shared__ __align__(16) BatchDesc sd;
+    __shared__ __align__(16) BatchSample sd;
     __shared__ uint4 philox_tab[kPhiloxTab * NB4];
     __shared__ uint32_t cube_step[2 * kDMax];
 
@@ -54,9 +54,9 @@ vsample_batch_kernel(const __grid_constant__ BatchArgs a)
         const BatchState& B = a.st[seg.slot];
         const int2 now = ld_volatile_int2(&B.it);
         {
-            const uint32_t* src = reinterpret_cast<const uint32_t*>(a.desc + seg.slot);
+            const uint32_t* src = reinterpret_cast<const uint32_t*>(static_cast<const BatchSample*>(a.desc + seg.slot));
             uint32_t* dst = reinterpret_cast<uint32_t*>(&sd);
-            for (uint32_t i = threadIdx.x; i < sizeof(BatchDesc) / 4; i += blockDim.x) dst[i] = src[i];
+            for (uint32_t i = threadIdx.x; i < sizeof(BatchSample) / 4; i += blockDim.x) dst[i] = src[i];
         }
         HT* hist = reinterpret_cast<HT*>(smem + (MIXED ? 0u : cell_bytes(false) * D * a.nb));
         Cell* cells = reinterpret_cast<Cell*>(smem + (MIXED ? hist_smem_bytes(true, D * a.nb) : 0u));
@@ -76,7 +76,7 @@ vsample_batch_kernel(const __grid_constant__ BatchArgs a)
         if (!run) continue;
         constexpr uint32_t d = D;
         const uint32_t nb = a.nb;
-        FamParams uf;  // single precision: the integrand's constants (those it reads)
+        FamConsts uf;  // single precision: the integrand's constants (those it reads)
         if constexpr (MIXED) {
 #pragma unroll
             for (int i = 0; i < kParMax; ++i) uf.cf[i] = uni(sd.fam.cf[i]);

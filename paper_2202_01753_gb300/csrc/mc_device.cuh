@@ -80,7 +80,7 @@ struct BatchView {
     float inv_p_f, inv_var_den_f;
     uint32_t want_abs;             // 0: a batch iteration does not use the sums of |cube mean|
     const uint32_t* cube_step;     // shared memory: [2][kDMax] digits of the cube step (cube_step_digit)
-    const FamParams& fam;
+    const FamConsts& fam;
 };
 
 // The keys grow by Weyl increments from the integral's own key.
@@ -418,7 +418,7 @@ template <bool kExact> __device__ __forceinline__ float bin_phi_f32(const BinPos
 
 // ---------------------------------------------------------------------------
 // Integrand families.  Each keeps a running state updated axis by axis, so
-// the point x never has to be stored; constants come from FamParams, whose
+// the point x never has to be stored; constants come from FamConsts, whose
 // layout per family is fixed by integrand_prepare (capi.cu):
 //   CONST    c[0] = v
 //   GAUSS    c[0] = A, c[1+j] = mu_j, c[13+j] = 1/(2 sig_j^2)
@@ -439,7 +439,7 @@ template <> struct RealOps<double> {
     __device__ static double log_(double v) { return fx::fx_log(v); }
     __device__ static double cos_(double v) { return cos(v); }
     __device__ static double rcp(double v) { return 1.0 / v; }
-    __device__ static double par(const FamParams& f, int i) { return f.c[i]; }
+    __device__ static double par(const FamConsts& f, int i) { return f.c[i]; }
 };
 template <> struct RealOps<float> {
     __device__ static float exp_(float v) { return expf(v); }
@@ -447,7 +447,7 @@ template <> struct RealOps<float> {
     __device__ static float log_(float v) { return logf(v); }
     __device__ static float cos_(float v) { return fx::fx_cosf(v); }
     __device__ static float rcp(float v) { return 1.0f / v; }
-    __device__ static float par(const FamParams& f, int i) { return f.cf[i]; }
+    __device__ static float par(const FamConsts& f, int i) { return f.cf[i]; }
 };
 
 template <int FAM, typename R> struct Family;
@@ -455,19 +455,19 @@ template <int FAM, typename R> struct Family;
 template <typename R> struct Family<MCUBES_F_CONST, R> {
     struct S {};
     __device__ static void begin(S&) {}
-    __device__ static void add(S&, int, R, const FamParams&) {}
-    __device__ static R end(const S&, uint32_t, const FamParams& f) { return RealOps<R>::par(f, 0); }
+    __device__ static void add(S&, int, R, const FamConsts&) {}
+    __device__ static R end(const S&, uint32_t, const FamConsts& f) { return RealOps<R>::par(f, 0); }
 };
 
 template <typename R> struct Family<MCUBES_F_GAUSS, R> {
     struct S { R q; };
     __device__ static void begin(S& s) { s.q = R(0); }
-    __device__ static void add(S& s, int j, R x, const FamParams& f)
+    __device__ static void add(S& s, int j, R x, const FamConsts& f)
     {
         const R z = x - RealOps<R>::par(f, 1 + j);
         s.q += z * z * RealOps<R>::par(f, 13 + j);
     }
-    __device__ static R end(const S& s, uint32_t, const FamParams& f)
+    __device__ static R end(const S& s, uint32_t, const FamConsts& f)
     {
         return RealOps<R>::par(f, 0) * RealOps<R>::expm_(s.q);
     }
@@ -476,8 +476,8 @@ template <typename R> struct Family<MCUBES_F_GAUSS, R> {
 template <typename R> struct Family<MCUBES_F_CORNER, R> {
     struct S { R t; };
     __device__ static void begin(S& s) { s.t = R(1); }
-    __device__ static void add(S& s, int j, R x, const FamParams& f) { s.t += RealOps<R>::par(f, j) * x; }
-    __device__ static R end(const S& s, uint32_t d, const FamParams&)
+    __device__ static void add(S& s, int j, R x, const FamConsts& f) { s.t += RealOps<R>::par(f, j) * x; }
+    __device__ static R end(const S& s, uint32_t d, const FamConsts&)
     {
         // t^-(d+1) by repeated squaring of 1/t
         R b = RealOps<R>::rcp(s.t), r = R(1);
@@ -494,8 +494,8 @@ template <typename R> struct Family<MCUBES_F_CORNER, R> {
 template <typename R> struct Family<MCUBES_F_OSC, R> {
     struct S { R t; };
     __device__ static void begin(S& s) { s.t = R(0); }
-    __device__ static void add(S& s, int j, R x, const FamParams& f) { s.t += RealOps<R>::par(f, 1 + j) * x; }
-    __device__ static R end(const S& s, uint32_t, const FamParams& f)
+    __device__ static void add(S& s, int j, R x, const FamConsts& f) { s.t += RealOps<R>::par(f, 1 + j) * x; }
+    __device__ static R end(const S& s, uint32_t, const FamConsts& f)
     {
         return RealOps<R>::cos_(RealOps<R>::par(f, 0) + s.t);
     }
@@ -504,34 +504,34 @@ template <typename R> struct Family<MCUBES_F_OSC, R> {
 template <typename R> struct Family<MCUBES_F_PRODPEAK, R> {
     struct S { R v; };
     __device__ static void begin(S& s) { s.v = R(1); }
-    __device__ static void add(S& s, int j, R x, const FamParams& f)
+    __device__ static void add(S& s, int j, R x, const FamConsts& f)
     {
         const R z = x - RealOps<R>::par(f, 12 + j);
         s.v *= RealOps<R>::rcp(RealOps<R>::par(f, j) + z * z);
     }
-    __device__ static R end(const S& s, uint32_t, const FamParams&) { return s.v; }
+    __device__ static R end(const S& s, uint32_t, const FamConsts&) { return s.v; }
 };
 
 template <typename R> struct Family<MCUBES_F_C0, R> {
     struct S { R t; };
     __device__ static void begin(S& s) { s.t = R(0); }
-    __device__ static void add(S& s, int j, R x, const FamParams& f)
+    __device__ static void add(S& s, int j, R x, const FamConsts& f)
     {
         const R z = x - RealOps<R>::par(f, 12 + j);
         s.t += RealOps<R>::par(f, j) * (z < R(0) ? -z : z);
     }
-    __device__ static R end(const S& s, uint32_t, const FamParams&) { return RealOps<R>::expm_(s.t); }
+    __device__ static R end(const S& s, uint32_t, const FamConsts&) { return RealOps<R>::expm_(s.t); }
 };
 
 template <typename R> struct Family<MCUBES_F_DISCONT, R> {
     struct S { R t; bool out; };
     __device__ static void begin(S& s) { s.t = R(0); s.out = false; }
-    __device__ static void add(S& s, int j, R x, const FamParams& f)
+    __device__ static void add(S& s, int j, R x, const FamConsts& f)
     {
         s.out |= !(x < RealOps<R>::par(f, 12 + j));
         s.t += RealOps<R>::par(f, j) * x;
     }
-    __device__ static R end(const S& s, uint32_t, const FamParams&)
+    __device__ static R end(const S& s, uint32_t, const FamConsts&)
     {
         return s.out ? R(0) : RealOps<R>::exp_(s.t);
     }
@@ -557,7 +557,7 @@ template <typename R> struct Family<MCUBES_F_COSMO6, R> {
     static constexpr bool kRolled = kWide;
     struct S { R e; R x12; };
     __device__ static void begin(S& s) { s.e = R(0); s.x12 = R(0); }
-    __device__ static void add(S& s, int j, R x, const FamParams& f)
+    __device__ static void add(S& s, int j, R x, const FamConsts& f)
     {
         const R L = RealOps<R>::log_(x);
         if constexpr (kWide) {
@@ -574,14 +574,14 @@ template <typename R> struct Family<MCUBES_F_COSMO6, R> {
         if (j == 0) s.x12 = x;
         if (j == 1) s.x12 += x;
     }
-    __device__ static R end(const S& s, uint32_t, const FamParams& f)
+    __device__ static R end(const S& s, uint32_t, const FamConsts& f)
     {
         const R z = s.x12 - RealOps<R>::par(f, 8);
         if constexpr (kWide) return RealOps<R>::expm_(s.e + z * z * f.c[9]);  // c10: in the Jacobian
         else return RealOps<R>::par(f, 10) * RealOps<R>::expm_(s.e + z * z * RealOps<R>::par(f, 9));
     }
     // f J in double precision, J = (jm / 2^63) 2^je the integer Jacobian
-    __device__ static double end_scaled(const S& s, const FamParams& f, uint64_t jm, int je)
+    __device__ static double end_scaled(const S& s, const FamConsts& f, uint64_t jm, int je)
     {
         const double z = s.x12 - f.c[8];
         return fx::fx_exp_neg_scaled(s.e + z * z * f.c[9], jm, je);
@@ -748,9 +748,9 @@ struct FixSum {
 template <> struct FixFamily<MCUBES_F_GAUSS> {
     static constexpr bool kHas = true;
     using S = FixSum;
-    __device__ static void begin(S& s, const FamParams& f) { s.q = f.fu[kDMax]; }
-    __device__ static void add(S& s, int, int64_t t, const FamParams&) { s.q += sq_fixed(t); }
-    template <int D> __device__ static double end(const S& s, const FamParams& f, const IntProd& jp)
+    __device__ static void begin(S& s, const FamConsts& f) { s.q = f.fu[kDMax]; }
+    __device__ static void add(S& s, int, int64_t t, const FamConsts&) { s.q += sq_fixed(t); }
+    template <int D> __device__ static double end(const S& s, const FamConsts& f, const IntProd& jp)
     {
         return fx::fx_exp_fixed<true>(s.q, f.fq, jp.m, jp.e);
     }
@@ -759,10 +759,10 @@ template <> struct FixFamily<MCUBES_F_GAUSS> {
 template <> struct FixFamily<MCUBES_F_C0> {
     static constexpr bool kHas = true;
     using S = FixSum;
-    __device__ static void begin(S& s, const FamParams& f) { s.q = f.fu[kDMax]; }
+    __device__ static void begin(S& s, const FamConsts& f) { s.q = f.fu[kDMax]; }
     // |t|, or one less on the negative side: t is cut downwards, so both sides are short by half a unit on average
-    __device__ static void add(S& s, int, int64_t t, const FamParams&) { s.q += (uint64_t)(t ^ (t >> 63)); }
-    template <int D> __device__ static double end(const S& s, const FamParams& f, const IntProd& jp)
+    __device__ static void add(S& s, int, int64_t t, const FamConsts&) { s.q += (uint64_t)(t ^ (t >> 63)); }
+    template <int D> __device__ static double end(const S& s, const FamConsts& f, const IntProd& jp)
     {
         return fx::fx_exp_fixed<true>(s.q, f.fq, jp.m, jp.e);
     }
@@ -774,17 +774,17 @@ template <> struct FixFamily<MCUBES_F_DISCONT> {
         uint64_t q;
         bool out;
     };
-    __device__ static void begin(S& s, const FamParams& f)
+    __device__ static void begin(S& s, const FamConsts& f)
     {
         s.q = f.fu[kDMax];
         s.out = false;
     }
-    __device__ static void add(S& s, int j, int64_t t, const FamParams& f)
+    __device__ static void add(S& s, int j, int64_t t, const FamConsts& f)
     {
         s.out |= (uint64_t)t >= f.fu[j];
         s.q += (uint64_t)t;
     }
-    template <int D> __device__ static double end(const S& s, const FamParams& f, const IntProd& jp)
+    template <int D> __device__ static double end(const S& s, const FamConsts& f, const IntProd& jp)
     {
         return s.out ? 0.0 : fx::fx_exp_fixed<false>(s.q, f.fq, jp.m, jp.e);
     }
@@ -793,9 +793,9 @@ template <> struct FixFamily<MCUBES_F_DISCONT> {
 template <> struct FixFamily<MCUBES_F_CORNER> {
     static constexpr bool kHas = true;
     using S = FixSum;
-    __device__ static void begin(S& s, const FamParams& f) { s.q = f.fu[kDMax]; }
-    __device__ static void add(S& s, int, int64_t t, const FamParams&) { s.q += (uint64_t)t; }
-    template <int D> __device__ static double end(const S& s, const FamParams& f, const IntProd& jp)
+    __device__ static void begin(S& s, const FamConsts& f) { s.q = f.fu[kDMax]; }
+    __device__ static void add(S& s, int, int64_t t, const FamConsts&) { s.q += (uint64_t)t; }
+    template <int D> __device__ static double end(const S& s, const FamConsts& f, const IntProd& jp)
     {
         // t^-(D+1) J by repeated squaring of 1/t
         IntProd b = int_prod_recip(int_prod_of_fixed(s.q, f.fq)), r = jp;
@@ -811,9 +811,9 @@ template <> struct FixFamily<MCUBES_F_CORNER> {
 template <> struct FixFamily<MCUBES_F_OSC> {
     static constexpr bool kHas = true;
     using S = FixSum;
-    __device__ static void begin(S& s, const FamParams& f) { s.q = f.fu[kDMax]; }
-    __device__ static void add(S& s, int, int64_t t, const FamParams&) { s.q += (uint64_t)t; }
-    template <int D> __device__ static double end(const S& s, const FamParams& f, const IntProd& jp)
+    __device__ static void begin(S& s, const FamConsts& f) { s.q = f.fu[kDMax]; }
+    __device__ static void add(S& s, int, int64_t t, const FamConsts&) { s.q += (uint64_t)t; }
+    template <int D> __device__ static double end(const S& s, const FamConsts& f, const IntProd& jp)
     {
         bool neg;
         const uint64_t v = fx::fx_cos_turns(s.q << (64 - f.fq), &neg);
@@ -826,13 +826,13 @@ template <> struct FixFamily<MCUBES_F_OSC> {
 template <> struct FixFamily<MCUBES_F_PRODPEAK> {
     static constexpr bool kHas = true;
     using S = IntProd;
-    __device__ static void begin(S& s, const FamParams&) { s = IntProd{1ull << 63, 0}; }
-    __device__ static void add(S& s, int j, int64_t t, const FamParams& f)
+    __device__ static void begin(S& s, const FamConsts&) { s = IntProd{1ull << 63, 0}; }
+    __device__ static void add(S& s, int j, int64_t t, const FamConsts& f)
     {
         // the squares are cut, by half a last place on average: every other axis takes one back
         s = int_prod_mul2(s, int_prod_of_fixed((1ull << f.fq) + (uint64_t)(j & 1) + sq_fixed(t), f.fq));
     }
-    template <int D> __device__ static double end(const S& s, const FamParams&, const IntProd& jp)
+    template <int D> __device__ static double end(const S& s, const FamConsts&, const IntProd& jp)
     {
         return int_prod_value(int_prod_mul2(jp, int_prod_recip(s)));
     }

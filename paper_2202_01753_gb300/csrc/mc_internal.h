@@ -76,21 +76,23 @@ constexpr int kTabFactorsMax = 10;
 
 // Integrand constants in the form the kernels use (derived on the host from
 // the public params blob, see integrand_prepare in capi.cu).
-struct FamParams {
+struct FamConsts {
     double c[kParMax];
     float cf[kParMax];
-    // TABLE family: factor q reads table tid[q] at axes a[q] (and b[q] >= 0)
-    int nf;
-    int tid[kTabFactorsMax], ta[kTabFactorsMax], tb[kTabFactorsMax];
-    const TableDesc* tabs;   // device array of the context's tables
     // fixed-point form of the FP64 affine families (affine_prepare in affine.cu):
     // 0 where it does not apply
     int fix;
     int fsg;                 // left shift that brings g phi's numerator (< g 2^33) to the top of 64 bits
-    int ftsh[kDMax];         // axis j: a cell width of binary exponent e moves the product right by ftsh[j] - e
     int fq;                  // fraction bits of the integrand's running sum
-    int ff[kDMax];           // TABLE: fraction bits of axis j
+    int ftsh[kDMax];         // axis j: a cell width of binary exponent e moves the product right by ftsh[j] - e
     uint64_t fu[kDMax + 1];  // DISCONT: thresholds; [kDMax]: start of the running sum
+};
+// With those of the TABLE family: factor q reads table tid[q] at axes ta[q] (and tb[q] >= 0).
+struct FamParams : FamConsts {
+    int nf;
+    int tid[kTabFactorsMax], ta[kTabFactorsMax], tb[kTabFactorsMax];
+    const TableDesc* tabs;   // device array of the context's tables
+    int ff[kDMax];           // fraction bits of axis j in the fixed-point form
 };
 
 // Cells of the fixed-point form: coordinate t = a + b x (x the unit-cube edge)
@@ -144,8 +146,11 @@ struct VsArgs {
 // Batched iterations (many independent integrals per launch)
 // ---------------------------------------------------------------------------
 
-// One resident integral of a batch, as the batched kernels read it.
-struct BatchDesc {
+// One resident integral of a batch, as the batched sampling kernels read it:
+// each block copies this part into static shared memory, which with the cells
+// and histogram of the largest grids (12 axes of 803 bins in FP64, 231264
+// bytes) has to stay within the 227 KB of a block.
+struct BatchSample {
     uint32_t d, nb, g, gmagic;
     uint32_t p, lanes;
     uint32_t key0, key1;        // Philox key = the integral's own seed
@@ -156,9 +161,14 @@ struct BatchDesc {
     float phi_scale_f;          // 1 / (g nb)
     float inv_p_f, inv_var_den_f;
     float pad2;
+    FamConsts fam;
+};
+static_assert(sizeof(BatchSample) <= 704, "beside 480 bytes of the batched kernel's own");
+
+// With what the refinement reads.
+struct BatchDesc : BatchSample {
     double lo[kDMax];
     double scale[kDMax];
-    FamParams fam;
     CellMap cm;                 // fam.fix: the cells' coordinates
     double* grid;               // [d][nb] edge high parts, then [d][nb] low parts
     void* cells;                // [d][nb] map cells of the grid (double2 in FP64, float2 in mixed), rebuilt
