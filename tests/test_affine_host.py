@@ -69,3 +69,16 @@ def test_mean_error(affine, case, power):
     d = len(params) if fid == CO else len(params) // 2
     _, err, err_double = affine("mean", fid, params, [0.0] * d, [1.0] * d, n=60000, power=power)
     assert abs(err) <= max(2.0 ** -52, abs(err_double))
+
+
+def test_selection_at_the_limits(affine):
+    """The cases that test_gpu_affine_limits.py runs take the fixed-point form, with the fraction bits that
+    their rule ends at; just outside it is not taken."""
+    from test_gpu_affine_limits import INSIDE
+    bits = dict(gauss=52, osc=57, c0=54, corner=56, prodpeak=52, discont=54)
+    for name, fid, params, d in INSIDE:
+        assert affine("fix", fid, params, [0.0] * d, [1.0] * d) == [1, bits[name.split("_")[0]]], name
+    for fid, params in ((W.F_GAUSS, [1.0, 0.0, 1.0 / (2.0 * 4100.0) ** 0.5]), (W.F_OSC, [0.3, 2.0 * np.pi * 65.0]),
+                        (W.F_C0, [513.0, 0.0]), (W.F_CORNER, [128.0]), (W.F_PRODPEAK, [64.0, 0.0]),
+                        (W.F_DISCONT, [513.0, 0.9])):
+        assert affine("fix", fid, params, [0.0], [1.0])[0] == 0, (fid, params)
