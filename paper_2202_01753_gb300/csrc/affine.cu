@@ -81,14 +81,14 @@ long long to_fixed(HD v, int f)  // v 2^f rounded, |v| 2^f < 2^63
 // family's slopes 300 put the mean off by 5-9e-16 relative).  An axis's whole
 // range of t is below 2^(63 - f), so that a cell of any width has a product
 // shift of at least 0.  Rules per family:
-//   GAUSS    sum of the largest t^2 < 2^12 (unit of the exponent 2^-52)
+//   GAUSS    sum of the largest t^2 < 2^12 (unit of the exponent 2^-52), an axis's range < 2^6
 //   C0       sum of the largest |t| < 2^9 (2^-54)
 //   DISCONT  the same, and a cut inside the box at t >= 2^55 units (the threshold
 //            and a sample's t are within three: less than the last place of
 //            x, where the double-precision form puts it)
 //   CORNER   largest sum < 2^12, and 1 + a.lo >= 2^56 units: the power d + 1
 //            multiplies the sum's relative error (from 1, sums below 128)
-//   PRODPEAK 1 + t^2 < 2^12 per axis
+//   PRODPEAK 1 + t^2 < 2^12 and the range < 2^6 per axis
 //   OSC      at most 2^6 turns per axis
 //   TABLE    every axis read by one table dimension at most
 void affine_prepare(int id, const double* params, int d, const double* lo, const double* scale, long long g, int nb,

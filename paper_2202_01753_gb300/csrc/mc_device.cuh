@@ -303,7 +303,7 @@ __device__ __forceinline__ double2 map_cell_f64(DD left, DD right, double lo, do
 }
 
 // Map cell of the fixed-point form, in integers: (t at the left edge as an
-// integer with 51 to 62 fraction bits, rounded to nearest, and t width / g as a double).
+// integer in units of 2^-f, rounded to nearest, and t width / g as a double).
 __device__ __forceinline__ double2 map_cell_fix(DD left, DD right, const CellMap& m, int j)
 {
     const int E = exponent_of(right.hi);
@@ -722,8 +722,9 @@ template <typename R> struct Family<MCUBES_F_TABLE, R> {
 // warp instructions per sample.  Adjusting passes of 9.65e6 samples at d = 6,
 // before and with this form: GAUSS 779 -> 392 us, CORNER 676 -> 357, OSC (f_A)
 // 781 -> 336, PRODPEAK 1224 -> 420, C0 879 -> 366, DISCONT 651 -> 360; what is
-// left on the FP64 pipe is the histogram's additions.  t_j's error is 2^-f absolute, f =
-// 57..63 (affine.cu keeps the range of t_j small enough for that, or the
+// left on the FP64 pipe is the histogram's additions.  t_j's error is about 2^-f
+// absolute, f at least 57 (C0 and DISCONT 54, CORNER such that the sum is 2^56
+// units or more; affine.cu keeps the ranges small enough for that, or the
 // double-precision form is used): below the rounding of x itself.
 // Scales: GAUSS t = (x - mu)/(sigma sqrt 2), sum of t^2; C0 t = c (x - w),
 // sum of |t|; DISCONT, CORNER t = a (x - lo); OSC t = a x / (2 pi) in turns,
@@ -844,7 +845,7 @@ template <> struct FixFamily<MCUBES_F_PRODPEAK> {
 // fetched before the first is used (random 8-byte reads of tables larger than
 // the caches: the fetches overlap instead of following one another).
 // table6 at 1e8 calls: 9.50 -> 7.98 ms per pass (FP64 pipe 80% busy before, 46
-// warp instructions per sample; now 34, and 4.8 TB/s from HBM, 70% of the
+// warp instructions per sample; now 38.7, and 5.0 TB/s from HBM, 74% of the
 // measured copy rate).  128 registers, 16 warps per SM: 20 and 24 warps with
 // spills measured 8.55 and 9.16 ms.
 template <> struct FixFamily<MCUBES_F_TABLE> {

@@ -26,12 +26,18 @@ constexpr int kVsThreadsMax = 1024; // largest block of a single-integral sampli
 // The FP64 six-axis kernel (62 registers) runs one block of 1024 threads per
 // SM: measured 8.19 ms per 1e8-call pass against 8.39 (2 x 512), 8.54
 // (2 x 448), 8.94 (3 x 320), 8.92 (3 x 288) and 8.79 ms (3 x 256).
+// The other FP64 kernels take up to 80-85 registers, so 24 warps are resident
+// however they are grouped, unless shared memory (24 bytes per axis and bin)
+// holds fewer blocks: three of 256 threads fit up to d = 6 at the default 500
+// bins, two from d = 7 on (384 threads each), one from d = 10 on (768;
+// oscillatory d = 12 at 1e7 calls 892 us a pass with 256 threads, 589 with 768).
+// With fewer bins the grouping makes no difference to the warps.
 constexpr int kCosmo6Threads = 1024;
 __host__ __device__ constexpr int vsample_threads(int family, bool mixed, int d)
 {
     if (mixed || family == MCUBES_F_TABLE) return kVsThreads;
     if (family == MCUBES_F_COSMO6) return d == 6 ? kCosmo6Threads : kVsThreads;
-    return d <= 6 ? kVsThreads : d <= 6 ? 256 : d <= 9 ? 384 : 768;
+    return d <= 6 ? kVsThreads : d <= 9 ? 384 : 768;
 }
 constexpr int kRefineThreads = 512;
 
@@ -96,8 +102,8 @@ struct FamParams : FamConsts {
 };
 
 // Cells of the fixed-point form: coordinate t = a + b x (x the unit-cube edge)
-// with fbits[j] fraction bits (on = 0: cells in the box's coordinates); a, b as such
-// integers, b / g as bg_m 2^(bg_e - 63).  Sums wrap around 2^64 (OSC: t in
+// in units of 2^-f, f the axis's fraction bits (on = 0: cells in the box's
+// coordinates); a, b in those units, b / g as bg_m 2^(bg_e - 63).  Sums wrap around 2^64 (OSC: t in
 // turns, whole ones do not matter).
 struct CellMap {
     long long a[kDMax];
